@@ -167,29 +167,16 @@ extern "C" int adjoint_shot(const sgb_grid *g, const float *velocity, const floa
         (rc = to_dev(wavelet, (size_t)nt * 4, (void **)&d_wav)) ||
         (rc = to_dev(observed, (size_t)nt * nrec * 4, (void **)&d_obs)))
         return rc;
-    // CFL against the model's maximum
-    int *d_range;
-    if ((rc = sc.get((void **)&d_range, 16))) return rc;
-    int init[4] = {0, 0x7f7fffff, 0, 0};
-    CUDA_TRY(cudaMemcpyAsync(d_range, init, sizeof init, cudaMemcpyHostToDevice, st));
-    vel_range_kernel<<<ew_grid(ncomp, *ds), 256, 0, st>>>(d_vel, ncomp, d_range);
-    CUDA_TRY(cudaGetLastError());
-    int range[4];
-    CUDA_TRY(cudaMemcpyAsync(range, d_range, sizeof range, cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(cudaStreamSynchronize(st));
-    if (range[2] != 0) return fail(SGB_ERR_INVALID_ARG, "velocity has non-positive or non-finite values");
-    float vmax_model;
-    memcpy(&vmax_model, &range[0], 4);
-    if ((double)g->dt > cfl_limit(g, vmax_model))
-        return fail(SGB_ERR_UNSTABLE_DT, "dt %g above the CFL limit %g of the model", (double)g->dt,
-                    cfl_limit(g, vmax_model));
+    // m, and the CFL check against the model's maximum
+    float *m;
+    if ((rc = sc.get((void **)&m, fbytes)) || (rc = make_model(g, L, st, sc, d_vel, m))) return rc;
     // fields
-    float *u0, *u1, *phi, *m, *w0, *w1, *mu0, *mu1, *gsum, *ck, *seg, *d_tr;
+    float *u0, *u1, *phi, *w0, *w1, *mu0, *mu1, *gsum, *ck, *seg, *d_tr;
     double *gsum64, *d_J;
     long long *d_off;
     int *d_err;  // this call's device error word: concurrent calls stay independent
     if ((rc = sc.get((void **)&u0, fbytes)) || (rc = sc.get((void **)&u1, fbytes)) ||
-        (rc = sc.get((void **)&phi, fbytes)) || (rc = sc.get((void **)&m, fbytes)) ||
+        (rc = sc.get((void **)&phi, fbytes)) ||
         (rc = sc.get((void **)&w0, fbytes)) || (rc = sc.get((void **)&w1, fbytes)) ||
         (rc = sc.get((void **)&mu0, fbytes)) || (rc = sc.get((void **)&mu1, fbytes)) ||
         (rc = sc.get((void **)&gsum, fbytes)) ||
@@ -201,12 +188,10 @@ extern "C" int adjoint_shot(const sgb_grid *g, const float *velocity, const floa
         return rc;
     CUDA_TRY(cudaMemsetAsync(d_err, 0, sizeof(int), st));
     CUDA_TRY(cudaMemcpyAsync(d_off, off.data(), (size_t)nrec * 8, cudaMemcpyHostToDevice, st));
-    for (float *f : {u0, u1, phi, m, w0, w1, mu0, mu1, gsum})
+    for (float *f : {u0, u1, phi, w0, w1, mu0, mu1, gsum})
         CUDA_TRY(cudaMemsetAsync(f, 0, fbytes, st));
     CUDA_TRY(cudaMemsetAsync(gsum64, 0, (size_t)L.elems * 8, st));
     CUDA_TRY(cudaMemsetAsync(d_J, 0, 8, st));
-    make_m_kernel<<<ew_grid(ncomp, *ds), 256, 0, st>>>(pad_geom(L), d_vel, g->dt, m);
-    CUDA_TRY(cudaGetLastError());
 
     StepArgs base;
     fill_step_constants(g, L, base);

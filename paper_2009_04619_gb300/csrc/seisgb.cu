@@ -392,6 +392,50 @@ PadGeom pad_geom(const sgb_layout_info &L)
     return pg;
 }
 
+// Grid of a layout-conversion launch: items of one plane in x, planes in y.
+dim3 conv_grid(long long plane_items, int planes)
+{
+    return dim3((unsigned)((plane_items + CONV_ITEMS - 1) / CONV_ITEMS),
+                (unsigned)std::min(planes, 65535));
+}
+
+// Whether rows of a compact array can be moved as quads.
+bool quad_rows(const sgb_layout_info &L, const void *compact, const void *padded)
+{
+    return L.Nx % 4 == 0 && aligned16(compact) && aligned16(padded);
+}
+
+// compact fp32 -> padded T; M: velocity -> m = (v dt)^2 (range: see to_padded_kernel).
+template <class T, bool M = false>
+cudaError_t enqueue_to_padded(const sgb_layout_info &L, const float *src, T *dst, cudaStream_t st,
+                              float dt = 0.0f, int *range = nullptr)
+{
+    if (quad_rows(L, src, dst))
+        to_padded_kernel<T, 4, M><<<conv_grid(L.stride_z / 4, (int)L.sz), CONV_THREADS, 0, st>>>(
+            pad_geom(L), src, dst, dt, range);
+    else
+        to_padded_kernel<T, 1, M><<<conv_grid(L.stride_z, (int)L.sz), CONV_THREADS, 0, st>>>(
+            pad_geom(L), src, dst, dt, range);
+    ++t_launches;
+    return cudaGetLastError();
+}
+
+// padded T -> compact fp32, times *scale (null: 1).
+template <class T>
+cudaError_t enqueue_from_padded(const sgb_layout_info &L, const T *src, const float *scale, float *dst,
+                                cudaStream_t st)
+{
+    const long long plane = (long long)L.Nx * L.Ny;
+    if (quad_rows(L, dst, src))
+        from_padded_kernel<T, 4><<<conv_grid(plane / 4, L.Nz), CONV_THREADS, 0, st>>>(pad_geom(L), src,
+                                                                                     scale, dst);
+    else
+        from_padded_kernel<T, 1><<<conv_grid(plane, L.Nz), CONV_THREADS, 0, st>>>(pad_geom(L), src,
+                                                                                 scale, dst);
+    ++t_launches;
+    return cudaGetLastError();
+}
+
 int ew_grid(long long n, const DevState &ds)
 {
     long long b = (n + 255) / 256;
@@ -527,9 +571,7 @@ extern "C" int sgb_pack(const sgb_grid *g, const float *compact, float *padded, 
     DevState *ds;
     if ((rc = device_state(&ds))) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    pack_kernel<<<ew_grid(L.elems, *ds), 256, 0, st>>>(pad_geom(L), compact, padded, L.elems);
-    CUDA_TRY(cudaGetLastError());
-    ++t_launches;
+    CUDA_TRY(enqueue_to_padded(L, compact, padded, st));
     return SGB_OK;
 }
 
@@ -542,10 +584,7 @@ extern "C" int sgb_unpack(const sgb_grid *g, const float *padded, float *compact
     DevState *ds;
     if ((rc = device_state(&ds))) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    unpack_kernel<<<ew_grid((long long)L.Nx * L.Ny * L.Nz, *ds), 256, 0, st>>>(pad_geom(L), padded,
-                                                                               compact);
-    CUDA_TRY(cudaGetLastError());
-    ++t_launches;
+    CUDA_TRY(enqueue_from_padded(L, padded, nullptr, compact, st));
     return SGB_OK;
 }
 
@@ -1045,7 +1084,7 @@ template <class T, bool DIFF = false>
 // device compact fp32 arrays (u^n, u^{n-1}, phi^n) read at n_begin and
 // overwritten with the state at n_end.  Traces rows are steps n_begin ...
 int run_shot_t(const sgb_grid *g, const sgb_layout_info &L, DevState *ds, cudaStream_t st,
-               Scratch &sc, const float *d_vel, const float *d_wav, int n_begin, int n_end,
+               Scratch &sc, const float *m, const float *d_wav, int n_begin, int n_end,
                const int32_t *src_ijk, const int32_t *rec_ijk, int nrec, const long long *d_off,
                float *d_tr, float *final_u, float *const *state, int *d_err)
 {
@@ -1054,34 +1093,27 @@ int run_shot_t(const sgb_grid *g, const sgb_layout_info &L, DevState *ds, cudaSt
     const long long ncomp = (long long)L.Nx * L.Ny * L.Nz;
     const size_t ubytes = (size_t)L.elems * sizeof(T), fbytes = (size_t)L.elems * 4;
     void *u0, *u1;
-    float *phi, *m;
+    float *phi;
     ScaleState *ss = nullptr;
     int *d_step;
     void *dfield = nullptr;  // difference form: d^n = u^n - u^{n-1}, updated in place
     if ((rc = sc.get(&u0, ubytes)) || (rc = sc.get(&u1, ubytes)) ||
-        (rc = sc.get((void **)&phi, fbytes)) || (rc = sc.get((void **)&m, fbytes)) ||
-        (rc = sc.get((void **)&d_step, sizeof(int))))
+        (rc = sc.get((void **)&phi, fbytes)) || (rc = sc.get((void **)&d_step, sizeof(int))))
         return rc;
     if (DIFF) {
         if ((rc = sc.get(&dfield, ubytes))) return rc;
         CUDA_TRY(cudaMemsetAsync(dfield, 0, ubytes, st));
     }
     CUDA_TRY(cudaMemcpyAsync(d_step, &n_begin, sizeof(int), cudaMemcpyHostToDevice, st));
-    CUDA_TRY(cudaMemsetAsync(m, 0, fbytes, st));
     if (!state) {
         CUDA_TRY(cudaMemsetAsync(u0, 0, ubytes, st));
         CUDA_TRY(cudaMemsetAsync(u1, 0, ubytes, st));
         CUDA_TRY(cudaMemsetAsync(phi, 0, fbytes, st));
     } else {  // u^n into buf[(n+1)&1], u^{n-1} into buf[n&1] (n = n_begin), phi^n
         void *bb[2] = {u0, u1};
-        const int eg = ew_grid(L.elems, *ds);
-        pack_t_kernel<T><<<eg, 256, 0, st>>>(pad_geom(L), state[0], static_cast<T *>(bb[(n_begin + 1) & 1]),
-                                             L.elems);
-        pack_t_kernel<T><<<eg, 256, 0, st>>>(pad_geom(L), state[1], static_cast<T *>(bb[n_begin & 1]),
-                                             L.elems);
-        pack_kernel<<<eg, 256, 0, st>>>(pad_geom(L), state[2], phi, L.elems);
-        CUDA_TRY(cudaGetLastError());
-        t_launches += 3;
+        CUDA_TRY(enqueue_to_padded(L, state[0], static_cast<T *>(bb[(n_begin + 1) & 1]), st));
+        CUDA_TRY(enqueue_to_padded(L, state[1], static_cast<T *>(bb[n_begin & 1]), st));
+        CUDA_TRY(enqueue_to_padded(L, state[2], phi, st));
     }
     ScaleState *ssd = nullptr;  // difference form: the scales of d
     if (Elem<T>::SCALED) {
@@ -1093,9 +1125,6 @@ int run_shot_t(const sgb_grid *g, const sgb_layout_info &L, DevState *ds, cudaSt
             CUDA_TRY(cudaMemcpyAsync(ssd, &init, sizeof init, cudaMemcpyHostToDevice, st));
         }
     }
-    make_m_kernel<<<ew_grid(ncomp, *ds), 256, 0, st>>>(pad_geom(L), d_vel, g->dt, m);
-    CUDA_TRY(cudaGetLastError());
-    ++t_launches;
 
     // buf[0] holds u^{-1}, buf[1] holds u^0; step n reads buf[(n+1)&1] and
     // overwrites buf[n&1] with u^{n+1}.
@@ -1197,22 +1226,15 @@ int run_shot_t(const sgb_grid *g, const sgb_layout_info &L, DevState *ds, cudaSt
         ++t_launches;
     }
     if (state) {  // the state at n_end: u^{nt}, u^{nt-1}, phi^{nt}
-        unpack_t_kernel<T><<<ew_grid(ncomp, *ds), 256, 0, st>>>(pad_geom(L),
-            static_cast<const T *>(u_final_dev), s_final, state[0]);
-        unpack_t_kernel<T><<<ew_grid(ncomp, *ds), 256, 0, st>>>(pad_geom(L),
-            static_cast<const T *>(buf[nt & 1]), nullptr, state[1]);
-        unpack_kernel<<<ew_grid(ncomp, *ds), 256, 0, st>>>(pad_geom(L), phi, state[2]);
-        CUDA_TRY(cudaGetLastError());
-        t_launches += 3;
+        CUDA_TRY(enqueue_from_padded(L, static_cast<const T *>(u_final_dev), s_final, state[0], st));
+        CUDA_TRY(enqueue_from_padded(L, static_cast<const T *>(buf[nt & 1]), nullptr, state[1], st));
+        CUDA_TRY(enqueue_from_padded(L, phi, nullptr, state[2], st));
     }
     if (final_u) {
         const bool host_u = !is_device_ptr(final_u);
         float *dst = final_u;
         if (host_u && (rc = sc.get((void **)&dst, (size_t)ncomp * 4))) return rc;
-        unpack_t_kernel<T><<<ew_grid(ncomp, *ds), 256, 0, st>>>(
-            pad_geom(L), static_cast<const T *>(u_final_dev), s_final, dst);
-        CUDA_TRY(cudaGetLastError());
-        ++t_launches;
+        CUDA_TRY(enqueue_from_padded(L, static_cast<const T *>(u_final_dev), s_final, dst, st));
         if (host_u)
             CUDA_TRY(cudaMemcpyAsync(final_u, dst, (size_t)ncomp * 4, cudaMemcpyDeviceToHost, st));
     }
@@ -1223,7 +1245,7 @@ int run_shot_t(const sgb_grid *g, const sgb_layout_info &L, DevState *ds, cudaSt
 // odd last step as one ordinary fused step.  Four wavefield buffers: a pair
 // reads (u^{n-1}, u^n) from one two and writes (u^{n+1}, u^{n+2}) to the other.
 int run_shot_pairs(const sgb_grid *g, const sgb_layout_info &L, DevState *ds, cudaStream_t st,
-                   Scratch &sc, const float *d_vel, const float *d_wav, int nt,
+                   Scratch &sc, const float *m, const float *d_wav, int nt,
                    const int32_t *src_ijk, int nrec, const long long *d_off, float *d_tr,
                    float *final_u, int *d_err)
 {
@@ -1231,20 +1253,15 @@ int run_shot_pairs(const sgb_grid *g, const sgb_layout_info &L, DevState *ds, cu
     if ((rc = prepare_two_step())) return rc;
     const long long ncomp = (long long)L.Nx * L.Ny * L.Nz;
     const size_t fbytes = (size_t)L.elems * 4;
-    float *u[4], *phi, *m;
+    float *u[4], *phi;
     int *d_step;
     for (int q = 0; q < 4; ++q)
         if ((rc = sc.get((void **)&u[q], fbytes))) return rc;
-    if ((rc = sc.get((void **)&phi, fbytes)) || (rc = sc.get((void **)&m, fbytes)) ||
-        (rc = sc.get((void **)&d_step, sizeof(int))))
+    if ((rc = sc.get((void **)&phi, fbytes)) || (rc = sc.get((void **)&d_step, sizeof(int))))
         return rc;
     CUDA_TRY(cudaMemsetAsync(d_step, 0, sizeof(int), st));
     for (int q = 0; q < 2; ++q) CUDA_TRY(cudaMemsetAsync(u[q], 0, fbytes, st));
     CUDA_TRY(cudaMemsetAsync(phi, 0, fbytes, st));
-    CUDA_TRY(cudaMemsetAsync(m, 0, fbytes, st));
-    make_m_kernel<<<ew_grid(ncomp, *ds), 256, 0, st>>>(pad_geom(L), d_vel, g->dt, m);
-    CUDA_TRY(cudaGetLastError());
-    ++t_launches;
 
     StepArgs base;
     fill_step_constants(g, L, base);
@@ -1340,9 +1357,7 @@ int run_shot_pairs(const sgb_grid *g, const sgb_layout_info &L, DevState *ds, cu
         const bool host_u = !is_device_ptr(final_u);
         float *dst = final_u;
         if (host_u && (rc = sc.get((void **)&dst, (size_t)ncomp * 4))) return rc;
-        unpack_kernel<<<ew_grid(ncomp, *ds), 256, 0, st>>>(pad_geom(L), u_final_dev, dst);
-        CUDA_TRY(cudaGetLastError());
-        ++t_launches;
+        CUDA_TRY(enqueue_from_padded(L, u_final_dev, nullptr, dst, st));
         if (host_u)
             CUDA_TRY(cudaMemcpyAsync(final_u, dst, (size_t)ncomp * 4, cudaMemcpyDeviceToHost, st));
     }
@@ -1416,6 +1431,34 @@ extern "C" int stencil_step2(const sgb_grid *g, const float *u_prev, const float
 
 namespace {
 
+// Status of a model whose range to_padded_kernel found: its values, and the CFL
+// check against its actual maximum.
+int check_model_range(const sgb_grid *g, const int (&range)[4])
+{
+    if (range[2] != 0) return fail(SGB_ERR_INVALID_ARG, "velocity has non-positive or non-finite values");
+    float vmax_model;
+    memcpy(&vmax_model, &range[0], 4);
+    if ((double)g->dt > cfl_limit(g, vmax_model))
+        return fail(SGB_ERR_UNSTABLE_DT, "dt %g above the CFL limit %g of the model (vmax %g)",
+                    (double)g->dt, cfl_limit(g, vmax_model), (double)vmax_model);
+    return SGB_OK;
+}
+
+// m = (v dt)^2 into a padded field and the model's range in the same pass, then
+// the checks (waits for the stream).
+int make_model(const sgb_grid *g, const sgb_layout_info &L, cudaStream_t st, Scratch &sc,
+               const float *d_vel, float *m)
+{
+    int *d_range, rc;
+    if ((rc = sc.get((void **)&d_range, 4 * sizeof(int)))) return rc;
+    int range[4] = {0, 0x7f7fffff, 0, 0};
+    CUDA_TRY(cudaMemcpyAsync(d_range, range, sizeof range, cudaMemcpyHostToDevice, st));
+    CUDA_TRY((enqueue_to_padded<float, true>(L, d_vel, m, st, g->dt, d_range)));
+    CUDA_TRY(cudaMemcpyAsync(range, d_range, sizeof range, cudaMemcpyDeviceToHost, st));
+    CUDA_TRY(cudaStreamSynchronize(st));
+    return check_model_range(g, range);
+}
+
 // run_shot and run_shot_segment: steps n_begin .. n_end-1; state (u^n,
 // u^{n-1}, phi^n compact fp32, host or device) or null for zero fields and no
 // state out.
@@ -1473,23 +1516,9 @@ int run_shot_common(const sgb_grid *g, const float *velocity, const float *wavel
         CUDA_TRY(cudaMemcpyAsync(t, velocity, cb, cudaMemcpyHostToDevice, st));
         d_vel = t;
     }
-    // velocity range -> CFL check against the model's actual maximum
-    int *d_range;
-    if ((rc = sc.get((void **)&d_range, 4 * sizeof(int)))) return rc;
-    int init[4] = {0, 0x7f7fffff, 0, 0};
-    CUDA_TRY(cudaMemcpyAsync(d_range, init, sizeof init, cudaMemcpyHostToDevice, st));
-    vel_range_kernel<<<ew_grid(ncomp, *ds), 256, 0, st>>>(d_vel, ncomp, d_range);
-    CUDA_TRY(cudaGetLastError());
-    ++t_launches;
-    int range[4];
-    CUDA_TRY(cudaMemcpyAsync(range, d_range, sizeof range, cudaMemcpyDeviceToHost, st));
-    CUDA_TRY(cudaStreamSynchronize(st));
-    if (range[2] != 0) return fail(SGB_ERR_INVALID_ARG, "velocity has non-positive or non-finite values");
-    float vmax_model;
-    memcpy(&vmax_model, &range[0], 4);
-    if ((double)g->dt > cfl_limit(g, vmax_model))
-        return fail(SGB_ERR_UNSTABLE_DT, "dt %g above the CFL limit %g of the model (vmax %g)",
-                    (double)g->dt, cfl_limit(g, vmax_model), (double)vmax_model);
+    float *m;
+    if ((rc = sc.get((void **)&m, (size_t)L.elems * 4))) return rc;
+    if ((rc = make_model(g, L, st, sc, d_vel, m))) return rc;
 
     const float *d_wav = wavelet;
     if (wavelet && nt > 0 && !is_device_ptr(wavelet)) {
@@ -1524,33 +1553,33 @@ int run_shot_common(const sgb_grid *g, const float *velocity, const float *wavel
     float *const *dst = state ? d_state : nullptr;
     switch (g->storage) {
     case SGB_FP16_SCALED:
-        rc = run_shot_t<__half>(g, L, ds, st, sc, d_vel, d_wav, n_begin, n_end, src_ijk, rec_ijk,
+        rc = run_shot_t<__half>(g, L, ds, st, sc, m, d_wav, n_begin, n_end, src_ijk, rec_ijk,
                                 nrec, d_off, d_tr, final_u, dst, d_err);
         break;
     case SGB_BF16:
-        rc = run_shot_t<__nv_bfloat16>(g, L, ds, st, sc, d_vel, d_wav, n_begin, n_end, src_ijk,
+        rc = run_shot_t<__nv_bfloat16>(g, L, ds, st, sc, m, d_wav, n_begin, n_end, src_ijk,
                                        rec_ijk, nrec, d_off, d_tr, final_u, dst, d_err);
         break;
     case SGB_FP32_DIFF:
-        rc = run_shot_t<float, true>(g, L, ds, st, sc, d_vel, d_wav, n_begin, n_end, src_ijk,
+        rc = run_shot_t<float, true>(g, L, ds, st, sc, m, d_wav, n_begin, n_end, src_ijk,
                                      rec_ijk, nrec, d_off, d_tr, final_u, dst, d_err);
         break;
     case SGB_BF16_DIFF:
-        rc = run_shot_t<__nv_bfloat16, true>(g, L, ds, st, sc, d_vel, d_wav, n_begin, n_end,
+        rc = run_shot_t<__nv_bfloat16, true>(g, L, ds, st, sc, m, d_wav, n_begin, n_end,
                                              src_ijk, rec_ijk, nrec, d_off, d_tr, final_u, dst,
                                              d_err);
         break;
     case SGB_FP16_DIFF:
-        rc = run_shot_t<__half, true>(g, L, ds, st, sc, d_vel, d_wav, n_begin, n_end, src_ijk,
+        rc = run_shot_t<__half, true>(g, L, ds, st, sc, m, d_wav, n_begin, n_end, src_ijk,
                                       rec_ijk, nrec, d_off, d_tr, final_u, dst, d_err);
         break;
     default:
         // temporal blocking covers whole shots; a segment takes one step per launch
         if (g->schedule == SGB_SCHED_PAIRS && !state && n_begin == 0)
-            rc = run_shot_pairs(g, L, ds, st, sc, d_vel, d_wav, nt, src_ijk, nrec, d_off, d_tr,
+            rc = run_shot_pairs(g, L, ds, st, sc, m, d_wav, nt, src_ijk, nrec, d_off, d_tr,
                                 final_u, d_err);
         else
-            rc = run_shot_t<float>(g, L, ds, st, sc, d_vel, d_wav, n_begin, n_end, src_ijk, rec_ijk,
+            rc = run_shot_t<float>(g, L, ds, st, sc, m, d_wav, n_begin, n_end, src_ijk, rec_ijk,
                                    nrec, d_off, d_tr, final_u, dst, d_err);
     }
     if (rc) return rc;
@@ -1707,27 +1736,16 @@ extern "C" int run_shot_noalloc(const sgb_grid *g, const float *velocity, const 
     long long *d_off = (long long *)(base + off_rec);
     int *d_range = (int *)(base + off_range);
     int *d_err = d_range + 4;  // this entry point's own error word
-    const int ewg = (int)std::min<long long>((ncomp + 255) / 256, (long long)ns->sms * 8);
 
     // the array keeps the previous call's contents: clear what must start at zero
-    CUDA_TRY(cudaMemsetAsync(base, 0, off_ijk, st));  // u0, u1, phi, m
+    CUDA_TRY(cudaMemsetAsync(base, 0, off_m, st));  // u0, u1, phi (m is written whole below)
     int init[8] = {0, 0x7f7fffff, 0, 0, 0, 0, 0, 0};  // velocity range; error word = 0
     CUDA_TRY(cudaMemcpyAsync(d_range, init, sizeof init, cudaMemcpyHostToDevice, st));
-    vel_range_kernel<<<ewg, 256, 0, st>>>(velocity, ncomp, d_range);
-    CUDA_TRY(cudaGetLastError());
-    ++t_launches;
+    CUDA_TRY((enqueue_to_padded<float, true>(L, velocity, m, st, g->dt, d_range)));
     int range[4];
     CUDA_TRY(cudaMemcpyAsync(range, d_range, sizeof range, cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
-    if (range[2] != 0) return fail(SGB_ERR_INVALID_ARG, "velocity has non-positive or non-finite values");
-    float vmax_model;
-    memcpy(&vmax_model, &range[0], 4);
-    if ((double)g->dt > cfl_limit(g, vmax_model))
-        return fail(SGB_ERR_UNSTABLE_DT, "dt %g above the CFL limit %g of the model (vmax %g)",
-                    (double)g->dt, cfl_limit(g, vmax_model), (double)vmax_model);
-    make_m_kernel<<<ewg, 256, 0, st>>>(pad_geom(L), velocity, g->dt, m);
-    CUDA_TRY(cudaGetLastError());
-    ++t_launches;
+    if ((rc = check_model_range(g, range))) return rc;
     if (nrec > 0) {
         CUDA_TRY(cudaMemcpyAsync(d_ijk, rec_ijk, (size_t)nrec * 12, cudaMemcpyHostToDevice, st));
         rec_offsets_kernel<<<(nrec + 255) / 256, 256, 0, st>>>(d_ijk, nrec, L.sx, L.stride_z,
@@ -1771,9 +1789,7 @@ extern "C" int run_shot_noalloc(const sgb_grid *g, const float *velocity, const 
         ++t_launches;
     }
     if (final_u) {
-        unpack_kernel<<<ewg, 256, 0, st>>>(pad_geom(L), u_last, final_u);
-        CUDA_TRY(cudaGetLastError());
-        ++t_launches;
+        CUDA_TRY(enqueue_from_padded(L, u_last, nullptr, final_u, st));
     }
     int dev_err = 0;
     CUDA_TRY(cudaMemcpyAsync(&dev_err, d_err, sizeof(int), cudaMemcpyDeviceToHost, st));

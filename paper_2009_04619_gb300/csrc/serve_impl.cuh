@@ -166,10 +166,7 @@ int setup_shot(sgb_server *sv, Shot *sh)
     CUDA_TRY(cudaMemsetAsync(sh->u0, 0, fbytes, st));
     CUDA_TRY(cudaMemsetAsync(sh->u1, 0, fbytes, st));
     CUDA_TRY(cudaMemsetAsync(sh->phi, 0, fbytes, st));
-    CUDA_TRY(cudaMemsetAsync(sh->m, 0, fbytes, st));
-    make_m_kernel<<<ew_grid(ncomp, *sv->ds), 256, 0, st>>>(pad_geom(L), sh->d_vel, sh->g.dt, sh->m);
-    CUDA_TRY(cudaGetLastError());
-    ++t_launches;
+    CUDA_TRY((enqueue_to_padded<float, true>(L, sh->d_vel, sh->m, st, sh->g.dt)));
     // the pageable copies above are staged before they return; wait for them so
     // the host copies can be released
     CUDA_TRY(cudaStreamSynchronize(st));
