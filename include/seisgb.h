@@ -78,7 +78,7 @@ typedef struct {
 
 /* run_shot time-loop schedules (the arithmetic per point is the same in all):
  *  SGB_SCHED_AUTO   the library's choice (SGB_SCHED_STEP, measured fastest);
- *  SGB_SCHED_STEP   one launch per step, replayed in CUDA graphs of 32 steps;
+ *  SGB_SCHED_STEP   one launch per step;
  *  SGB_SCHED_PAIRS  temporal blocking: two steps per pass over HBM on the
  *                   PML-free interior, see stencil_step2 (SGB_FP32 only);
  *  SGB_SCHED_FLOW   one persistent launch for the whole time loop: CTAs take
@@ -278,7 +278,7 @@ int adjoint_shot(const sgb_grid *g, const float *velocity, const float *wavelet,
  *    there); calls whose GPU work overlaps, on any streams, race on it and give
  *    wrong results or statuses;
  *  - like run_shot, outputs that overlap an input or each other are rejected;
- *  - the time loop is launched directly, one kernel per step (no CUDA graph). */
+ *  - the time loop is one launch per step, whatever the schedule. */
 int run_shot_noalloc(const sgb_grid *g, const float *velocity, const float *wavelet, int32_t nt,
                      const int32_t *src_ijk, const int32_t *rec_ijk, int32_t nrec, float *traces,
                      float *final_u, void *stream);

@@ -169,12 +169,14 @@ extern "C" int adjoint_shot(const sgb_grid *g, const float *velocity, const floa
         return rc;
     // m, and the CFL check against the model's maximum
     float *m;
-    if ((rc = sc.get((void **)&m, fbytes)) || (rc = make_model(g, L, st, sc, d_vel, m))) return rc;
+    int *d_range, *d_err;  // d_err: this call's device error word, so concurrent calls stay independent
+    if ((rc = get_call_words(sc, st, &d_range, &d_err)) || (rc = sc.get((void **)&m, fbytes)) ||
+        (rc = make_model(g, L, st, d_vel, m, d_range)))
+        return rc;
     // fields
     float *u0, *u1, *phi, *w0, *w1, *mu0, *mu1, *gsum, *ck, *seg, *d_tr;
     double *gsum64, *d_J;
     long long *d_off;
-    int *d_err;  // this call's device error word: concurrent calls stay independent
     if ((rc = sc.get((void **)&u0, fbytes)) || (rc = sc.get((void **)&u1, fbytes)) ||
         (rc = sc.get((void **)&phi, fbytes)) ||
         (rc = sc.get((void **)&w0, fbytes)) || (rc = sc.get((void **)&w1, fbytes)) ||
@@ -184,9 +186,8 @@ extern "C" int adjoint_shot(const sgb_grid *g, const float *velocity, const floa
         (rc = sc.get((void **)&seg, fbytes * (size_t)C)) ||
         (rc = sc.get((void **)&d_tr, (size_t)nt * nrec * 4)) ||
         (rc = sc.get((void **)&gsum64, (size_t)L.elems * 8)) || (rc = sc.get((void **)&d_J, 8)) ||
-        (rc = sc.get((void **)&d_off, (size_t)nrec * 8)) || (rc = sc.get((void **)&d_err, 16)))
+        (rc = sc.get((void **)&d_off, (size_t)nrec * 8)))
         return rc;
-    CUDA_TRY(cudaMemsetAsync(d_err, 0, sizeof(int), st));
     CUDA_TRY(cudaMemcpyAsync(d_off, off.data(), (size_t)nrec * 8, cudaMemcpyHostToDevice, st));
     for (float *f : {u0, u1, phi, w0, w1, mu0, mu1, gsum})
         CUDA_TRY(cudaMemsetAsync(f, 0, fbytes, st));

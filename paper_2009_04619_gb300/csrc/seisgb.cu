@@ -1,5 +1,5 @@
 // C-ABI host side of seisgb: validation, padded layout, TMA tensor maps,
-// launch configuration, CUDA-graph time loop (run_shot).
+// launch configuration, time loops.
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <cudaTypedefs.h>
@@ -267,6 +267,8 @@ bool in_inner(const sgb_grid *g, int i, int j, int k)
     return i >= g->nb && i < g->nb + g->nx && j >= g->nb && j < g->nb + g->ny && k >= g->nb &&
            k < g->nb + g->nz;
 }
+
+size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -1088,21 +1090,18 @@ int run_shot_t(const sgb_grid *g, const sgb_layout_info &L, DevState *ds, cudaSt
     void *u0, *u1;
     float *phi;
     ScaleState *ss = nullptr;
-    int *d_step;
     void *dfield = nullptr;  // difference form: d^n = u^n - u^{n-1}, updated in place
-    if ((rc = sc.get(&u0, ubytes)) || (rc = sc.get(&u1, ubytes)) ||
-        (rc = sc.get((void **)&phi, fbytes)) || (rc = sc.get((void **)&d_step, sizeof(int))))
-        return rc;
-    if (DIFF) {
-        if ((rc = sc.get(&dfield, ubytes))) return rc;
-        CUDA_TRY(cudaMemsetAsync(dfield, 0, ubytes, st));
+    {   // u^n, u^{n-1}, phi (and d) in one block, cleared at once
+        const size_t us = align256(ubytes), bytes = (DIFF ? 3 : 2) * us + fbytes;
+        unsigned char *block;
+        if ((rc = sc.get((void **)&block, bytes))) return rc;
+        u0 = block;
+        u1 = block + us;
+        if (DIFF) dfield = block + 2 * us;
+        phi = reinterpret_cast<float *>(block + (DIFF ? 3 : 2) * us);
+        if (!state) CUDA_TRY(cudaMemsetAsync(block, 0, bytes, st));
     }
-    CUDA_TRY(cudaMemcpyAsync(d_step, &n_begin, sizeof(int), cudaMemcpyHostToDevice, st));
-    if (!state) {
-        CUDA_TRY(cudaMemsetAsync(u0, 0, ubytes, st));
-        CUDA_TRY(cudaMemsetAsync(u1, 0, ubytes, st));
-        CUDA_TRY(cudaMemsetAsync(phi, 0, fbytes, st));
-    } else {  // u^n into buf[(n+1)&1], u^{n-1} into buf[n&1] (n = n_begin), phi^n
+    if (state) {  // u^n into buf[(n+1)&1], u^{n-1} into buf[n&1] (n = n_begin), phi^n
         void *bb[2] = {u0, u1};
         CUDA_TRY(enqueue_to_padded(L, state[0], static_cast<T *>(bb[(n_begin + 1) & 1]), st));
         CUDA_TRY(enqueue_to_padded(L, state[1], static_cast<T *>(bb[n_begin & 1]), st));
@@ -1154,15 +1153,6 @@ int run_shot_t(const sgb_grid *g, const sgb_layout_info &L, DevState *ds, cudaSt
                                       L)))
             return rc;
 
-    auto args_for = [&](int parity, const int *step_ptr, int step_add) {
-        StepArgs a = base;
-        a.u_out = buf[parity & 1];
-        a.u_cur = buf[(parity + 1) & 1];
-        a.step_ptr = step_ptr;
-        a.step_add = step_add;
-        return a;
-    };
-
     bool looped = false;
     if constexpr (!Elem<T>::SCALED && !DIFF) {
         if (resolve_schedule(g) == SGB_SCHED_FLOW && nsteps > 0) {
@@ -1171,42 +1161,19 @@ int run_shot_t(const sgb_grid *g, const sgb_layout_info &L, DevState *ds, cudaSt
             looped = true;
         }
     }
-    const int GS = 32;  // steps per graph replay (even: the buffer parity repeats)
-    const int replays = looped ? 0 : nsteps / GS;
-    if (replays > 0) {
-        cudaStream_t cs;
-        CUDA_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
-        cudaGraph_t graph = nullptr;
-        cudaGraphExec_t exec = nullptr;
-        int crc = SGB_OK;
-        cudaError_t ce = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
-        if (ce == cudaSuccess) {
-            for (int i = 0; i < GS && crc == SGB_OK; ++i)
-                crc = launch_step<T, DIFF>(args_for(n_begin + i, d_step, i), maps[(n_begin + i) & 1],
-                                           grid, cs);
-            if (crc == SGB_OK) {
-                advance_kernel<<<1, 32, 0, cs>>>(d_step, GS);
-                ce = cudaGetLastError();
-            }
-            cudaError_t ee = cudaStreamEndCapture(cs, &graph);
-            if (ce == cudaSuccess) ce = ee;
+    // One launch per step, straight onto the stream: with the programmatic
+    // dependency a step costs the host less than the smallest step takes on the
+    // GPU (3 against 6 us), so the queue stays full without graphs, whose capture
+    // and instantiation left the GPU idle at the start of every call (96^3 x 100
+    // steps: 955 -> 864 us; 1000 steps: the same within 1%).
+    if (!looped)
+        for (int n = n_begin; n < n_end; ++n) {
+            StepArgs a = base;
+            a.u_out = buf[n & 1];
+            a.u_cur = buf[(n + 1) & 1];
+            a.step_add = n;
+            if ((rc = launch_step<T, DIFF>(a, maps[n & 1], grid, st))) return rc;
         }
-        t_launches -= GS;  // captured launches are counted at replay
-        if (ce == cudaSuccess && crc == SGB_OK) ce = cudaGraphInstantiate(&exec, graph, 0);
-        if (ce == cudaSuccess && crc == SGB_OK) {
-            for (int r = 0; r < replays && ce == cudaSuccess; ++r) {
-                ce = cudaGraphLaunch(exec, st);
-                t_launches += GS + 1;
-            }
-        }
-        if (exec) cudaGraphExecDestroy(exec);
-        if (graph) cudaGraphDestroy(graph);
-        cudaStreamDestroy(cs);
-        if (crc) return crc;
-        CUDA_TRY(ce);
-    }
-    for (int n = looped ? n_end : n_begin + replays * GS; n < n_end; ++n)
-        if ((rc = launch_step<T, DIFF>(args_for(n, nullptr, n), maps[n & 1], grid, st))) return rc;
 
     // u^k lives in buf[(k+1)&1] (written by step k-1): u^{nt} in buf[(nt+1)&1]
     const void *u_final_dev = buf[(nt + 1) & 1];
@@ -1437,15 +1404,24 @@ int check_model_range(const sgb_grid *g, const int (&range)[4])
     return SGB_OK;
 }
 
+// Device words of one call: the model's range (as to_padded_kernel wants it) and
+// the call's own error word, in one allocation and one copy.
+int get_call_words(Scratch &sc, cudaStream_t st, int **d_range, int **d_err)
+{
+    int rc;
+    if ((rc = sc.get((void **)d_range, 8 * sizeof(int)))) return rc;
+    *d_err = *d_range + 4;
+    const int init[8] = {0, 0x7f7fffff, 0, 0, 0, 0, 0, 0};
+    CUDA_TRY(cudaMemcpyAsync(*d_range, init, sizeof init, cudaMemcpyHostToDevice, st));
+    return SGB_OK;
+}
+
 // m = (v dt)^2 into a padded field and the model's range in the same pass, then
 // the checks (waits for the stream).
-int make_model(const sgb_grid *g, const sgb_layout_info &L, cudaStream_t st, Scratch &sc,
-               const float *d_vel, float *m)
+int make_model(const sgb_grid *g, const sgb_layout_info &L, cudaStream_t st, const float *d_vel,
+               float *m, int *d_range)
 {
-    int *d_range, rc;
-    if ((rc = sc.get((void **)&d_range, 4 * sizeof(int)))) return rc;
-    int range[4] = {0, 0x7f7fffff, 0, 0};
-    CUDA_TRY(cudaMemcpyAsync(d_range, range, sizeof range, cudaMemcpyHostToDevice, st));
+    int range[4];
     CUDA_TRY((enqueue_to_padded<float, true>(L, d_vel, m, st, g->dt, d_range)));
     CUDA_TRY(cudaMemcpyAsync(range, d_range, sizeof range, cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
@@ -1499,9 +1475,8 @@ int run_shot_common(const sgb_grid *g, const float *velocity, const float *wavel
     cudaStream_t st = (cudaStream_t)stream;
 
     Scratch sc{st, ds->pool, {}};
-    int *d_err = nullptr;  // this call's own device error word
-    if ((rc = sc.get((void **)&d_err, sizeof(int)))) return rc;
-    CUDA_TRY(cudaMemsetAsync(d_err, 0, sizeof(int), st));
+    int *d_range, *d_err;  // ... and this call's own device error word
+    if ((rc = get_call_words(sc, st, &d_range, &d_err))) return rc;
     const float *d_vel = velocity;
     if (!is_device_ptr(velocity)) {
         float *t;
@@ -1511,7 +1486,7 @@ int run_shot_common(const sgb_grid *g, const float *velocity, const float *wavel
     }
     float *m;
     if ((rc = sc.get((void **)&m, (size_t)L.elems * 4))) return rc;
-    if ((rc = make_model(g, L, st, sc, d_vel, m))) return rc;
+    if ((rc = make_model(g, L, st, d_vel, m, d_range))) return rc;
 
     const float *d_wav = wavelet;
     if (wavelet && nt > 0 && !is_device_ptr(wavelet)) {
@@ -1669,8 +1644,6 @@ __global__ void rec_offsets_kernel(const int32_t *ijk, int nrec, long long sx, l
         off[r] = origin + (long long)ijk[3 * r + 2] * sxy + (long long)ijk[3 * r + 1] * sx +
                  ijk[3 * r];
 }
-
-size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
 }  // namespace
 
