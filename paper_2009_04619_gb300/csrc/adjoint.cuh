@@ -40,25 +40,9 @@ __global__ void fold_kernel(float *__restrict__ S, double *__restrict__ G, long 
     }
 }
 
-// Residual of step k-1 enters at the receivers: w^k += m r, and its term of
-// the gradient sum, S += (m r) g^{k-1}.
-__global__ void inject_residual_kernel(float *__restrict__ w, const float *__restrict__ m,
-                                       const float *__restrict__ acc, float *__restrict__ S,
-                                       const long long *__restrict__ rec_off, int nrec,
-                                       const float *__restrict__ traces_row,
-                                       const float *__restrict__ obs_row)
-{
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r < nrec) {
-        const long long p = rec_off[r];
-        const float add = m[p] * (traces_row[r] - obs_row[r]);
-        w[p] += add;
-        S[p] = fmaf(add, acc[p], S[p]);
-    }
-}
-
 // J = 1/2 sum (traces - observed)^2 in fp64, in a fixed order (two passes:
-// per-block partial sums, then one block), so repeated runs agree to the bit.
+// per-block partial sums, then one block of as many threads), so repeated runs
+// agree to the bit.
 constexpr int MISFIT_BLOCKS = 256;
 
 __global__ void misfit_partial_kernel(const float *__restrict__ tr, const float *__restrict__ obs,
@@ -81,25 +65,38 @@ __global__ void misfit_partial_kernel(const float *__restrict__ tr, const float 
     }
 }
 
-__global__ void misfit_final_kernel(const double *partial, int n, double *J)
+__global__ void misfit_final_kernel(const double *partial, double *J)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        double t = 0.0;
-        for (int b = 0; b < n; ++b) t += partial[b];
+    __shared__ double ws[MISFIT_BLOCKS / 32];
+    double t = partial[threadIdx.x];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = t;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        t = 0.0;
+        for (int w = 0; w < MISFIT_BLOCKS / 32; ++w) t += ws[w];
         *J = t;
     }
 }
 
-// dJ/dv = 2 (sum_k w^k g^{k-1}) / v on the compact grid.
+// dJ/dv = 2 (sum_k w^k g^{k-1}) / v on the compact grid, planes in grid.y.  fp64
+// division is slow here (87 us at 128^3): 1 / v comes from the fp32 reciprocal
+// and one Newton step in fp64 (relative error below 2^-46), the indices from one
+// 32-bit division.
 __global__ void chain_kernel(PadGeom g, const double *__restrict__ G,
                              const float *__restrict__ vel, double *__restrict__ grad_v)
 {
-    const long long n = (long long)g.Nx * g.Ny * g.Nz;
-    for (long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x; c < n;
-         c += (long long)gridDim.x * blockDim.x) {
-        const long long i = c % g.Nx, t = c / g.Nx;
-        const long long j = t % g.Ny, k = t / g.Ny;
-        grad_v[c] = 2.0 * G[g.origin + k * g.sxy + j * g.sx + i] / (double)vel[c];
+    const uint32_t items = uint32_t(g.Nx) * uint32_t(g.Ny);
+    for (int k = blockIdx.y; k < g.Nz; k += gridDim.y) {
+        const long long c0 = (long long)k * items, p0 = g.origin + k * g.sxy;
+        for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < items; t += gridDim.x * blockDim.x) {
+            const uint32_t j = t / uint32_t(g.Nx), i = t - j * uint32_t(g.Nx);
+            const float v = vel[c0 + t];
+            double inv = (double)__frcp_rn(v);
+            inv = fma(inv, fma(-(double)v, inv, 1.0), inv);
+            if (!(v > 1e-30f && v < 1e30f)) inv = 1.0 / (double)v;  // no fp32 reciprocal there
+            grad_v[c0 + t] = 2.0 * G[p0 + j * g.sx + i] * inv;
+        }
     }
 }
 
@@ -233,7 +230,7 @@ extern "C" int adjoint_shot(const sgb_grid *g, const float *velocity, const floa
     if ((rc = sc.get((void **)&d_part, MISFIT_BLOCKS * 8))) return rc;
     misfit_partial_kernel<<<MISFIT_BLOCKS, 256, 0, st>>>(d_tr, d_obs, (long long)nt * nrec, d_part);
     CUDA_TRY(cudaGetLastError());
-    misfit_final_kernel<<<1, 32, 0, st>>>(d_part, MISFIT_BLOCKS, d_J);
+    misfit_final_kernel<<<1, MISFIT_BLOCKS, 0, st>>>(d_part, d_J);
     CUDA_TRY(cudaGetLastError());
 
     // 2. backward sweep, segment by segment from the last
@@ -257,10 +254,34 @@ extern "C" int adjoint_shot(const sgb_grid *g, const float *velocity, const floa
     CUtensorMap gs_map;
     if ((rc = encode_map<float>(&gs_map, gsum, L, CfgAdj::BX, CfgAdj::BY))) return rc;
     StepArgs abase = base;
-    abase.sk = -1;  // the adjoint's sources are the receivers (injected separately)
+    abase.sk = -1;  // the adjoint's sources are the receivers
     abase.gsum = gsum;
     int agrid = 0;
     choose_decomposition(L.Nx, L.Ny, L.Nz, ds->sms, adjoint_occ, abase, &agrid);
+    // receivers grouped by the unit that computes them
+    UnitReceivers ur;
+    int *d_rs, *d_ri;
+    long long *d_ro;
+    group_receivers(abase, agrid, rec_ijk, nrec, ur);
+    std::vector<long long> uoff(nrec);
+    for (int q = 0; q < nrec; ++q) uoff[q] = off[ur.list[q]];
+    if ((rc = sc.get((void **)&d_rs, ur.start.size() * 4)) || (rc = sc.get((void **)&d_ri, (size_t)nrec * 4)) ||
+        (rc = sc.get((void **)&d_ro, (size_t)nrec * 8)))
+        return rc;
+    CUDA_TRY(cudaMemcpyAsync(d_rs, ur.start.data(), ur.start.size() * 4, cudaMemcpyHostToDevice, st));
+    CUDA_TRY(cudaMemcpyAsync(d_ri, ur.list.data(), (size_t)nrec * 4, cudaMemcpyHostToDevice, st));
+    CUDA_TRY(cudaMemcpyAsync(d_ro, uoff.data(), (size_t)nrec * 8, cudaMemcpyHostToDevice, st));
+    abase.rec_start = d_rs;
+    abase.rec_idx = d_ri;
+    abase.rec_off = d_ro;
+    abase.m_all = m;
+    for (int q = 0; q < 3; ++q) {
+        abase.rec_lo[q] = abase.rec_hi[q] = rec_ijk[q];
+        for (int r = 1; r < nrec; ++r) {
+            abase.rec_lo[q] = std::min(abase.rec_lo[q], rec_ijk[3 * r + q]);
+            abase.rec_hi[q] = std::max(abase.rec_hi[q], rec_ijk[3 * r + q]);
+        }
+    }
     const int fgrid = ew_grid(L.elems, *ds);
     for (int s = nseg - 1; s >= 0; --s) {
         const int na = s * C, nbnd = std::min(na + C, nt);
@@ -286,17 +307,16 @@ extern "C" int adjoint_shot(const sgb_grid *g, const float *velocity, const floa
             a.u_cur = wbuf[(k + 1) & 1];
             a.phi = mbuf[k & 1];
             a.mu_in = mbuf[(k + 1) & 1];
+            a.acc_in = seg + (size_t)(k - 1 - na) * L.elems;
+            a.tr_row = d_tr + (size_t)(k - 1) * nrec;
+            a.obs_row = d_obs + (size_t)(k - 1) * nrec;
             a.step_add = k;
             const StepMaps &mp = amaps[k & 1];
             CUDA_TRY(launch_dependent(adjoint_step_kernel<CfgAdj>, agrid, CfgAdj::BLOCK,
                                       Stage<CfgAdj, float, MODE_ADJ>::SMEM_BYTES, st, a, mp.ucur,
                                       mp.ucur_in, mp.uprev, mp.m, mp.phi, acc_maps[k - 1 - na],
                                       gs_map));
-            inject_residual_kernel<<<(nrec + 255) / 256, 256, 0, st>>>(
-                wbuf[k & 1], m, seg + (size_t)(k - 1 - na) * L.elems, gsum, d_off, nrec,
-                d_tr + (size_t)(k - 1) * nrec, d_obs + (size_t)(k - 1) * nrec);
-            CUDA_TRY(cudaGetLastError());
-            t_launches += 2;
+            ++t_launches;
             if ((k - 1) % FOLD_EVERY == 0) {  // blocks of steps counted from step 0
                 fold_kernel<<<fgrid, 256, 0, st>>>(gsum, gsum64, (long long)L.elems);
                 CUDA_TRY(cudaGetLastError());
@@ -308,7 +328,8 @@ extern "C" int adjoint_shot(const sgb_grid *g, const float *velocity, const floa
     double *d_gv = grad_velocity;
     const bool host_gv = !is_device_ptr(grad_velocity);
     if (host_gv && (rc = sc.get((void **)&d_gv, (size_t)ncomp * 8))) return rc;
-    chain_kernel<<<ew_grid(ncomp, *ds), 256, 0, st>>>(pad_geom(L), gsum64, d_vel, d_gv);
+    chain_kernel<<<conv_grid((long long)L.Nx * L.Ny, L.Nz), CONV_THREADS, 0, st>>>(pad_geom(L), gsum64,
+                                                                                 d_vel, d_gv);
     CUDA_TRY(cudaGetLastError());
     if (host_gv)
         CUDA_TRY(cudaMemcpyAsync(grad_velocity, d_gv, (size_t)ncomp * 8, cudaMemcpyDeviceToHost, st));

@@ -64,11 +64,6 @@ __device__ __forceinline__ void fence_proxy_async_global()
     asm volatile("fence.proxy.async.global;" ::: "memory");
 }
 
-__device__ __forceinline__ void consumer_barrier(int threads)
-{
-    asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
-}
-
 // A stored wavefield value read through L2 (not L1), as fp32.
 __device__ __forceinline__ float ld_cg_value(const float *p) { return __ldcg(p); }
 __device__ __forceinline__ float ld_cg_value(const __nv_bfloat16 *p)

@@ -101,6 +101,12 @@ __device__ __forceinline__ uint64_t policy_evict_last()
     return p;
 }
 
+// Barrier of a CTA's consumer threads (the producer warp takes no part).
+__device__ __forceinline__ void consumer_barrier(int threads)
+{
+    asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+}
+
 // Approximate reciprocal (the PTX rcp.approx instruction, about 1 ulp); used
 // for 1 / (1 + eta dt), whose argument lies in [1, 2].
 __device__ __forceinline__ float rcp_approx(float x)

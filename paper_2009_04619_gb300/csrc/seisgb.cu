@@ -997,6 +997,27 @@ int prepare_flow(int *occ)
     return SGB_OK;
 }
 
+// Receivers grouped by the work unit that computes them: those of unit u are
+// list[start[u]] .. list[start[u + 1] - 1], in the caller's order.
+struct UnitReceivers {
+    std::vector<int> start, list;
+};
+
+void group_receivers(const StepArgs &a, int units, const int32_t *rec_ijk, int nrec, UnitReceivers &ur)
+{
+    const int tiles = a.tiles_x * a.tiles_y;
+    ur.start.assign(units + 1, 0);
+    ur.list.assign(std::max(nrec, 1), 0);
+    auto unit_of = [&](int r) {
+        const int i = rec_ijk[3 * r], j = rec_ijk[3 * r + 1], k = rec_ijk[3 * r + 2];
+        return (k / a.zc) * tiles + (j / Cfg::BY) * a.tiles_x + i / Cfg::BX;
+    };
+    for (int r = 0; r < nrec; ++r) ++ur.start[unit_of(r) + 1];
+    for (int u = 0; u < units; ++u) ur.start[u + 1] += ur.start[u];
+    std::vector<int> pos(ur.start.begin(), ur.start.end() - 1);
+    for (int r = 0; r < nrec; ++r) ur.list[pos[unit_of(r)]++] = r;
+}
+
 // Steps 0 .. nt-1 of a shot in one persistent dataflow launch.  base: the step
 // constants with phi, error word, source and receivers; maps[p], buf: the
 // tensor maps and buffers of steps of parity p (step n writes buf[n & 1]).
@@ -1021,18 +1042,9 @@ int run_flow(const sgb_layout_info &L, DevState *ds, cudaStream_t st, Scratch &s
         if ((long long)tiles * ((L.Nz + fa.zc - 1) / fa.zc) >= 2LL * ctas) break;
     }
     const int chunks = (L.Nz + fa.zc - 1) / fa.zc, units = tiles * chunks;
-    // receivers grouped by the unit that computes them
-    std::vector<int> rs(units + 1, 0), rl(std::max(nrec, 1));
-    auto unit_of = [&](int r) {
-        const int i = rec_ijk[3 * r], j = rec_ijk[3 * r + 1], k = rec_ijk[3 * r + 2];
-        return (k / fa.zc) * tiles + (j / Cfg::BY) * fa.tiles_x + i / Cfg::BX;
-    };
-    for (int r = 0; r < nrec; ++r) ++rs[unit_of(r) + 1];
-    for (int u = 0; u < units; ++u) rs[u + 1] += rs[u];
-    {
-        std::vector<int> pos(rs.begin(), rs.end() - 1);
-        for (int r = 0; r < nrec; ++r) rl[pos[unit_of(r)]++] = r;
-    }
+    UnitReceivers ur;
+    group_receivers(fa, units, rec_ijk, nrec, ur);
+    const std::vector<int> &rs = ur.start, &rl = ur.list;
     int *d_done, *d_counter, *d_rs, *d_rl;
     if ((rc = sc.get((void **)&d_done, (size_t)units * 4)) || (rc = sc.get((void **)&d_counter, 16)) ||
         (rc = sc.get((void **)&d_rs, rs.size() * 4)) || (rc = sc.get((void **)&d_rl, rl.size() * 4)))

@@ -118,6 +118,14 @@ struct StepArgs {
     float *acc_out;        // MODE_FWD_ACC: g = L u^n + phi^n + f^n (padded fp32)
     float *gsum;           // MODE_ADJ: fp32 partial sum of w^k g^{k-1} (padded)
     const float *mu_in;    // MODE_ADJ: mu^{k+1} (padded); phi is mu^k
+    // MODE_ADJ: the residual of step k - 1 enters w^k at the receivers. rec_off
+    // then lists them grouped by the work unit that computes them: those of unit
+    // u are rec_start[u] .. rec_start[u + 1] - 1, receiver rec_idx[q] of the rows
+    // (rec_box: the points they lie in, bounds inclusive)
+    const int *rec_start, *rec_idx;
+    const float *tr_row, *obs_row;  // traces and observed samples of step k - 1
+    const float *m_all, *acc_in;    // m and g^{k-1} (padded)
+    int rec_lo[3], rec_hi[3];
     int *err;              // device error word
     int tiles_x, tiles_y, zc;
     // shell launches of a temporally blocked pair: work units (x0, y0, z0, z1)
@@ -1135,6 +1143,26 @@ __device__ __forceinline__ void step_unit(const StepArgs &a, int unit, int units
     float4 q[TY][C::QN];
     st.consume_unit(q);
 
+    if constexpr (MODE == MODE_ADJ) {
+        // Residuals of this unit's receivers, on top of what its threads have just
+        // written: w^k += m r and its term of the gradient sum, S += (m r) g^{k-1}.
+        // A launch of its own for them took 3.5 us per step and stood between two
+        // steps that otherwise overlap (128^3: 41 -> 37 us per step and its
+        // forward and recomputation steps).
+        if (st.x0 <= a.rec_hi[0] && st.x0 + BX > a.rec_lo[0] && st.y0 <= a.rec_hi[1] &&
+            st.y0 + BY > a.rec_lo[1] && st.z0 <= a.rec_hi[2] && st.z1 > a.rec_lo[2]) {
+            const int r0 = a.rec_start[unit], r1 = a.rec_start[unit + 1];
+            consumer_barrier(THREADS);
+            float *w = static_cast<float *>(a.u_out);
+            for (int q = r0 + tid; q < r1; q += THREADS) {
+                const long long p = a.rec_off[q];
+                const int r = a.rec_idx[q];
+                const float add = a.m_all[p] * (a.tr_row[r] - a.obs_row[r]);
+                w[p] = __ldcg(w + p) + add;
+                a.gsum[p] = fmaf(add, a.acc_in[p], __ldcg(a.gsum + p));
+            }
+        }
+    }
     if constexpr (S::SCALED) {  // max |u^{n+1}| for the next step's scale
         float v = st.vmax;
         for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
