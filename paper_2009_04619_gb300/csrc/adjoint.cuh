@@ -27,7 +27,7 @@
 
 namespace {
 
-using CfgAdj = TileCfg<SGB_TXT, SGB_TYT, SGB_TY, SGB_NU, 2, SGB_MINB, SGB_UNROLL>;
+using CfgAdj = TileCfg<SGB_TXT, SGB_TYT, SGB_TY, SGB_NU, 2, SGB_MINB>;
 constexpr int FOLD_EVERY = 32;
 
 // G += S, S = 0 over the padded arrays (the fp64 time sum of the gradient).

@@ -75,7 +75,7 @@ __device__ __forceinline__ float ld_cg_value(const __nv_bfloat16 *p)
 // Wait (the whole warp) until the units around `unit` have completed `need`
 // steps.  False when the wait gave up or another CTA did.
 __device__ __forceinline__ bool flow_wait_deps(const FlowArgs &f, int chunks, int unit, int need,
-                                               int *err, int *s_abort)
+                                               int *err, volatile int *s_abort)
 {
     if (need <= 0) return true;
     const int lane = threadIdx.x & 31;
@@ -96,10 +96,10 @@ __device__ __forceinline__ bool flow_wait_deps(const FlowArgs &f, int chunks, in
         if (lane == 0)
             give_up = global_timer_ns() - t0 > 2000000000ull ||
                       (*reinterpret_cast<volatile int *>(err) & DEV_ERR_TIMEOUT) ||
-                      *reinterpret_cast<volatile int *>(s_abort);
+                      *s_abort;
         if (__any_sync(0xffffffffu, give_up)) {
             if (lane == 0) {
-                *reinterpret_cast<volatile int *>(s_abort) = 1;
+                *s_abort = 1;
                 atomicOr(err, DEV_ERR_TIMEOUT);
             }
             return false;
@@ -129,47 +129,26 @@ __global__ void __launch_bounds__(C::BLOCK, (min_blocks<C, T>()))
     using S = StepCta<C, T, MODE_FWD, VAR_FLOW>;
     using G = Stage<C, T>;
     static_assert(!S::SCALED, "the dataflow launch has no per-step fp16 scale");
-    constexpr int NU = S::NU, NP = S::NP, THREADS = C::THREADS, TY = C::TY;
+    constexpr int THREADS = C::THREADS, TY = C::TY;
 
-    extern __shared__ __align__(128) unsigned char smem_raw[];
     S st;
-    st.su = smem_raw;
-    st.sp = smem_raw + NU * G::U_BYTES;
-    st.full_u = reinterpret_cast<uint64_t *>(st.sp + NP * G::P_BYTES + G::MZ_BYTES);
-    st.empty_u = st.full_u + NU;
-    st.full_p = st.empty_u + NU;
-    st.empty_p = st.full_p + NP;
-    st.lastf_u = reinterpret_cast<int *>(st.empty_p + NP);
-    st.lastf_p = st.lastf_u + NU;
-    st.s_abort = st.lastf_p + NP;
-    uint64_t *item_full = reinterpret_cast<uint64_t *>(smem_raw + (G::SMEM_BYTES + 7) / 8 * 8);
+    uint64_t *item_full = reinterpret_cast<uint64_t *>(step_smem + (G::SMEM_BYTES + 7) / 8 * 8);
     uint64_t *item_empty = item_full + 2;
     int *item_buf = reinterpret_cast<int *>(item_empty + 2);
 
     const int tid = threadIdx.x;
     st.tid = tid;
-    st.lane = tid & 31;
+
     st.aborted = false;
     st.s_cur = st.s_prev = st.inv_s_next = 1.0f;
     st.vmax = 0.0f;
-    st.useq = st.pseq = 0;
     st.tm_acc = st.tm_gs = nullptr;
     st.pa = &a0;
     const int chunks = (a0.Nz + a0.zc - 1) / a0.zc;
     const int total = (f.n_end - f.n_begin) * f.units;
 
     if (tid == THREADS) {
-        *st.s_abort = (*reinterpret_cast<volatile int *>(a0.err) & DEV_ERR_TIMEOUT) ? 1 : 0;
-        for (int i = 0; i < NU; ++i) {
-            mbar_init(st.full_u + i, 1);
-            mbar_init(st.empty_u + i, C::WARPS);
-            st.lastf_u[i] = -1;
-        }
-        for (int i = 0; i < NP; ++i) {
-            mbar_init(st.full_p + i, 1);
-            mbar_init(st.empty_p + i, C::WARPS);
-            st.lastf_p[i] = -1;
-        }
+        st.init_rings((*reinterpret_cast<volatile int *>(a0.err) & DEV_ERR_TIMEOUT) ? 1 : 0);
         for (int i = 0; i < 2; ++i) {
             mbar_init(item_full + i, 1);
             mbar_init(item_empty + i, C::WARPS);
@@ -177,7 +156,7 @@ __global__ void __launch_bounds__(C::BLOCK, (min_blocks<C, T>()))
         fence_barrier_init();
     }
     __syncthreads();
-    st.aborted = *reinterpret_cast<volatile int *>(st.s_abort) != 0;
+    st.aborted = *st.s_abort() != 0;
 
     auto place = [&](int item, int &n, int &unit) {
         n = f.n_begin + item / f.units;
@@ -194,7 +173,7 @@ __global__ void __launch_bounds__(C::BLOCK, (min_blocks<C, T>()))
     };
 
     if (tid >= THREADS) {  // producer warp: takes items, waits for them, issues copies
-        const int lane = st.lane;
+        const int lane = tid & 31;
         for (int k = 0;; ++k) {
             int item = 0;
             if (lane == 0) item = atomicAdd(f.counter, 1);
@@ -210,7 +189,7 @@ __global__ void __launch_bounds__(C::BLOCK, (min_blocks<C, T>()))
             if (stop) break;
             int n, unit;
             place(item, n, unit);
-            if (!flow_wait_deps(f, chunks, unit, n, a0.err, st.s_abort)) break;
+            if (!flow_wait_deps(f, chunks, unit, n, a0.err, st.s_abort())) break;
             if (lane == 0) {
                 __threadfence();
                 fence_proxy_async_global();
@@ -223,8 +202,6 @@ __global__ void __launch_bounds__(C::BLOCK, (min_blocks<C, T>()))
                 st.unit_geometry();
                 st.produce_unit();
             }
-            st.useq += st.z1 - st.z0 + 8;
-            st.pseq += st.z1 - st.z0;
             st.aborted = __shfl_sync(0xffffffffu, st.aborted ? 1 : 0, 0) != 0;
         }
         if (lane == 0) st.drain();
@@ -234,24 +211,21 @@ __global__ void __launch_bounds__(C::BLOCK, (min_blocks<C, T>()))
     float4 q[TY][C::QN];
     for (int k = 0;; ++k) {
         const int slot = k & 1;
-        st.wait(item_full + slot, (k >> 1) & 1);
+        st.wait_warp(item_full + slot, (k >> 1) & 1);
         const int item = *reinterpret_cast<volatile int *>(item_buf + slot);
         __syncwarp();
-        if (st.lane == 0) mbar_arrive(item_empty + slot);
-        st.aborted = st.aborted || *reinterpret_cast<volatile int *>(st.s_abort) != 0;
+        if ((tid & 31) == 0) mbar_arrive(item_empty + slot);
+        st.aborted = st.aborted || *st.s_abort() != 0;
         if (item < 0 || st.aborted) break;
         int n, unit;
         place(item, n, unit);
         st.unit_geometry();
         st.thread_geometry();
         st.consume_unit(q);
-        const int nit = st.z1 - st.z0;
         // the unit's last four u planes only fed the queue: release their slots
         __syncwarp();
-        if (st.lane == 0)
-            for (int s = 0; s < 4; ++s) mbar_arrive(st.empty_u + (st.useq + nit + 4 + s) % NU);
-        st.useq += nit + 8;
-        st.pseq += nit;
+        if ((tid & 31) == 0)
+            for (int s = 1; s <= 4; ++s) mbar_arrive(st.empty_u(st.uf.behind(s)));
         // unit complete: its receivers' samples of u^{n+1}, then the flag
         consumer_barrier(THREADS);
         const StepArgs &a = a0;
@@ -267,7 +241,7 @@ __global__ void __launch_bounds__(C::BLOCK, (min_blocks<C, T>()))
         consumer_barrier(THREADS);
         // after an abort the unit's results are incomplete: no flag, so that
         // the units waiting for it give up as well
-        if (tid == 0 && !*reinterpret_cast<volatile int *>(st.s_abort)) {
+        if (tid == 0 && !*st.s_abort()) {
             __threadfence();
             st_release_gpu(f.done + unit, n + 1);
         }

@@ -359,7 +359,7 @@ int encode_step_maps(StepMaps &mp, const void *u_cur, const void *u_prev, const 
     using G = Stage<Cfg, T>;
     int rc;
     if ((rc = encode_map<T>(&mp.ucur, u_cur, L, G::SW, Cfg::SH, SGB_L2PROMO))) return rc;
-    if ((rc = encode_map<T>(&mp.ucur_in, u_cur, L, Cfg::BX, Cfg::BY))) return rc;
+    if ((rc = encode_map<T>(&mp.ucur_in, u_cur, L, G::SW, Cfg::BY))) return rc;
     if ((rc = encode_map<T>(&mp.uprev, u_prev, L, Cfg::BX, Cfg::BY))) return rc;
     if ((rc = encode_map<float>(&mp.m, m, L, Cfg::BX, Cfg::BY))) return rc;
     if ((rc = encode_map<float>(&mp.phi, phi ? phi : m, L, Cfg::PHI_BW, Cfg::BY))) return rc;

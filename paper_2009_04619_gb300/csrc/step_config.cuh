@@ -19,9 +19,6 @@ namespace sgb {
 #ifndef SGB_TY
 #define SGB_TY 2
 #endif
-#ifndef SGB_UNROLL
-#define SGB_UNROLL 1
-#endif
 #ifndef SGB_NU
 #define SGB_NU 9
 #endif
@@ -43,7 +40,7 @@ namespace sgb {
 #ifndef SGB_L2PROMO_P
 #define SGB_L2PROMO_P CU_TENSOR_MAP_L2_PROMOTION_NONE
 #endif
-using Cfg = TileCfg<SGB_TXT, SGB_TYT, SGB_TY, SGB_NU, SGB_NP, SGB_MINB, SGB_UNROLL>;
+using Cfg = TileCfg<SGB_TXT, SGB_TYT, SGB_TY, SGB_NU, SGB_NP, SGB_MINB>;
 
 // Chunking of z: pick the chunk length that minimises waves x (chunk + priming
 // overhead) for the resident-CTA slots of this GPU.  Chunks are capped at 40

@@ -33,18 +33,29 @@
 //    to the producer, so there is no block-wide barrier in the z loop;
 //  - each thread owns 4 consecutive x points (128-bit accesses) in TY rows;
 //    the z-neighbours of its points sit in a register queue (the paper's
-//    register-streaming idea, section IV); the z loop is unrolled U times with
-//    compile-time queue offsets and the queue shifts by U once per group, so
-//    there are 8 register moves per U planes.  Full 9-fold unrolling (the
-//    paper's st_reg_fixed form, no moves at all) measured slower on GB300:
-//    its code no longer fits the instruction cache;
+//    register-streaming idea, section IV) that moves by one place per plane.
+//    Full 9-fold unrolling (the paper's st_reg_fixed form, no moves at all)
+//    measured slower on GB300: its code no longer fits the instruction cache.
+//    Partial sums that move with each multiply-add need no moves either, but
+//    lengthen the start of every chunk and spill in the PML planes;
 //  - whether a plane takes the PML path depends only on the tile and k, so
 //    the branch is uniform across the CTA: the z range of a tile splits into
 //    segments of three plane kinds (interior; PML path outside the z-PML, where
 //    1/(1+e) and 1-e come from per-thread tables; z-PML), each a separately
-//    compiled loop, which keeps the hot interior loop small enough for the
-//    instruction cache; inside a PML-path plane, inner points select the Eq. 2
+//    compiled loop, and compiled once; inside a PML-path plane, inner points select the Eq. 2
 //    result computed by the same instructions as the interior path, bit for bit;
+//  - what bounds it: two warps per scheduler run a plane's chain of about 330
+//    (interior) to 450 (PML) instructions each, DRAM at 84-92% of the measured
+//    copy rate beside them, so instructions count: ring positions are running
+//    offsets with the barriers at a fixed place in each slot, what a thread has
+//    to know about its points is one word of flags, both waits of a plane are
+//    polled at once, the x taps and the PML update are packed pairs, and each
+//    plane kind is compiled once (83 -> 46 KB of code).  Per step, before and
+//    after: 512^3 + PML 32 411 -> 403 us, 256^3 + PML 16 63.1 -> 61.5 us, 96^3
+//    7.6 -> 7.2 us; bf16 at 512^3 427 -> 399 us, fp16 at 384 x 384 x 256 143 -> 132
+//    us.  No register may spill: beside 2 x 113 KB of shared memory the L1 holds
+//    a few KB, and a spilled value read in the z loop comes from L2 (80 bytes of
+//    spills took 256^3 from 65 to 95 us);
 //  - eta and its central differences are evaluated in closed form from the
 //    integer depth into the layer: no eta array is read;
 //  - every mbarrier wait is bounded (2 s); on timeout the CTA records
@@ -179,9 +190,27 @@ __device__ __forceinline__ uint32_t cvt_rs_bf16x2(float lo, float hi, uint32_t r
     return d;
 }
 
+// The first n (1..3) of four fp32 values: the quad that crosses the grid's last
+// column. Straight-line predicated stores: a loop over n here made the tiles at
+// a ragged edge the slowest of the grid (343 columns: 81 us a step, 344: 62).
+__device__ __forceinline__ void st_part(float *p, const float4 &v, int n)
+{
+    if (n > 0) p[0] = v.x;
+    if (n > 1) p[1] = v.y;
+    if (n > 2) p[2] = v.z;
+}
+// The same of two words of packed 16-bit pairs.
+__device__ __forceinline__ void st_part16(void *p, const uint2 &r, int n)
+{
+    uint16_t *q = static_cast<uint16_t *>(p);
+    if (n > 0) q[0] = (uint16_t)r.x;
+    if (n > 1) q[1] = (uint16_t)(r.x >> 16);
+    if (n > 2) q[2] = (uint16_t)r.y;
+}
+
 // Storage traits: TMA x margin (16 bytes), 4-wide loads from shared memory and
-// stores to global memory (rnd: random bits for stochastic rounding), scalar
-// access.
+// stores to global memory (rnd: random bits for stochastic rounding; FULL: all
+// four values, else the first n), scalar reads.
 template <class T>
 struct Elem;
 
@@ -190,9 +219,13 @@ struct Elem<float> {
     static constexpr int HX = 4;
     static constexpr bool SCALED = false;
     __device__ static __forceinline__ float4 ld(const float *p) { return lds128(p); }
-    __device__ static __forceinline__ void st(float *p, float4 v, uint32_t) { stg128(p, v); }
+    template <bool FULL>
+    __device__ static __forceinline__ void st(float *p, float4 v, uint32_t, int n)
+    {
+        if (FULL) stg128(p, v);
+        else st_part(p, v, n);
+    }
     __device__ static __forceinline__ float get(const float *p) { return *p; }
-    __device__ static __forceinline__ void put(float *p, float v, uint32_t) { *p = v; }
 };
 
 template <>
@@ -216,20 +249,18 @@ struct Elem<__half> {
         return *reinterpret_cast<const __half2 *>(&d);
 #endif
     }
-    __device__ static __forceinline__ void st(__half *p, float4 v, uint32_t rnd)
+    template <bool FULL>
+    __device__ static __forceinline__ void st(__half *p, float4 v, uint32_t rnd, int n)
     {
         // the second pair's word: an odd multiple of the first (cheap, uniform)
         __half2 a = pack(v.x, v.y, rnd), b = pack(v.z, v.w, rnd * 0x9E3779B1u);
         uint2 r;
         r.x = *reinterpret_cast<uint32_t *>(&a);
         r.y = *reinterpret_cast<uint32_t *>(&b);
-        *reinterpret_cast<uint2 *>(p) = r;
+        if (FULL) *reinterpret_cast<uint2 *>(p) = r;
+        else st_part16(p, r, n);
     }
     __device__ static __forceinline__ float get(const __half *p) { return __half2float(*p); }
-    __device__ static __forceinline__ void put(__half *p, float v, uint32_t rnd)
-    {
-        *p = pack(v, v, rnd).x;
-    }
 };
 
 template <>
@@ -253,29 +284,26 @@ struct Elem<__nv_bfloat16> {
         return *reinterpret_cast<const __nv_bfloat162 *>(&d);
 #endif
     }
-    __device__ static __forceinline__ void st(__nv_bfloat16 *p, float4 v, uint32_t rnd)
+    template <bool FULL>
+    __device__ static __forceinline__ void st(__nv_bfloat16 *p, float4 v, uint32_t rnd, int n)
     {
         // the second pair's word: an odd multiple of the first (cheap, uniform)
         __nv_bfloat162 a = pack(v.x, v.y, rnd), b = pack(v.z, v.w, rnd * 0x9E3779B1u);
         uint2 r;
         r.x = *reinterpret_cast<uint32_t *>(&a);
         r.y = *reinterpret_cast<uint32_t *>(&b);
-        *reinterpret_cast<uint2 *>(p) = r;
+        if (FULL) *reinterpret_cast<uint2 *>(p) = r;
+        else st_part16(p, r, n);
     }
     __device__ static __forceinline__ float get(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
-    __device__ static __forceinline__ void put(__nv_bfloat16 *p, float v, uint32_t rnd)
-    {
-        *p = pack(v, v, rnd).x;
-    }
 };
 
 constexpr int align128(int b) { return (b + 127) / 128 * 128; }
 
-template <int TXT_, int TYT_, int TY_, int NU_, int NP_, int MINB_, int U_>
+template <int TXT_, int TYT_, int TY_, int NU_, int NP_, int MINB_>
 struct TileCfg {
     static constexpr int TXT = TXT_, TYT = TYT_, TY = TY_, NU = NU_, NP = NP_, MINB = MINB_;
-    static constexpr int U = U_;       // z-loop unroll factor
-    static constexpr int QN = 8 + U_;  // register-queue length
+    static constexpr int QN = 2 * R + 1;  // register-queue length
     static constexpr int THREADS = TXT * TYT;   // consumer (compute) threads
     static constexpr int BLOCK = THREADS + 32;  // plus one producer warp
     static constexpr int BX = 4 * TXT, BY = TY * TYT;
@@ -288,10 +316,14 @@ struct TileCfg {
     static constexpr int PHI_BW = 32, PHI_NB = BX / PHI_BW;
     static_assert(NU >= 8, "the u ring must hold the 8 planes that prime the register queue");
     static_assert(BX % PHI_BW == 0 && PHI_NB <= 8, "phi blocks");
-    static_assert(U_ >= 1 && U_ <= 9, "unroll factor");
+    static_assert(TY <= 2, "flag bits of a thread's rows");
     static_assert(NP >= 2 && THREADS % 32 == 0, "ring sizes");
     static_assert(SH <= 256 && BX <= 240 && BY <= 256, "TMA box limits");
 };
+
+// Dynamic shared memory of the step kernels (no static shared memory, so the TMA
+// destinations start at the aligned base).
+extern __shared__ __align__(128) unsigned char step_smem[];
 
 // Shared-memory geometry of a configuration for storage type T (bytes).
 template <class C, class T, int MODE = MODE_FWD>
@@ -320,9 +352,10 @@ struct Stage {
 #endif
     static constexpr int NU = sizeof(T) == 2 ? SGB_NU16 : C::NU;
     static constexpr int NP = sizeof(T) == 2 ? SGB_NP16 : C::NP;
-    static constexpr size_t SMEM_BYTES = size_t(NU) * U_BYTES + size_t(NP) * P_BYTES +
-                                         size_t(MZ_BYTES) + size_t(NU + NP) * 16 +
-                                         size_t(NU + NP + 1) * 4;
+    // a slot: its tiles, then its full and empty barriers
+    static constexpr int U_PITCH = U_BYTES + 128, P_PITCH = P_BYTES + 128;
+    static constexpr int MZ_OFF = NU * U_PITCH + NP * P_PITCH, ABORT_OFF = MZ_OFF + MZ_BYTES;
+    static constexpr size_t SMEM_BYTES = size_t(ABORT_OFF) + 8;
     static_assert(U_BYTES % 128 == 0 && F_BYTES % 128 == 0, "stage alignment");
     static_assert(SW <= 256, "TMA box limit");
 };
@@ -344,19 +377,6 @@ __device__ __forceinline__ void f4set(float4 &v, int e, float s)
     else if (e == 2) v.z = s;
     else v.w = s;
 }
-#ifdef SGB_SCALAR_FMA
-__device__ __forceinline__ void f4fma(float4 &acc, float c, const float4 &v)
-{
-    acc.x = fmaf(c, v.x, acc.x);
-    acc.y = fmaf(c, v.y, acc.y);
-    acc.z = fmaf(c, v.z, acc.z);
-    acc.w = fmaf(c, v.w, acc.w);
-}
-__device__ __forceinline__ float4 f4mul(float c, const float4 &v)
-{
-    return make_float4(c * v.x, c * v.y, c * v.z, c * v.w);
-}
-#else
 // acc += c * v on a float4 as two packed f32x2 FMAs.
 __device__ __forceinline__ void f4fma(float4 &acc, float c, const float4 &v)
 {
@@ -373,7 +393,67 @@ __device__ __forceinline__ float4 f4mul(float c, const float4 &v)
     float2 hi = __fmul2_rn(cc, make_float2(v.z, v.w));
     return make_float4(lo.x, lo.y, hi.x, hi.y);
 }
-#endif
+
+// a * b + c, a * b, a + b and a - b element by element: packed pairs, each
+// operation rounded once.
+__device__ __forceinline__ float4 f4fma4(const float4 &a, const float4 &b, const float4 &c)
+{
+    const float2 lo = __ffma2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y), make_float2(c.x, c.y));
+    const float2 hi = __ffma2_rn(make_float2(a.z, a.w), make_float2(b.z, b.w), make_float2(c.z, c.w));
+    return make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+__device__ __forceinline__ float4 f4mul4(const float4 &a, const float4 &b)
+{
+    const float2 lo = __fmul2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
+    const float2 hi = __fmul2_rn(make_float2(a.z, a.w), make_float2(b.z, b.w));
+    return make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+__device__ __forceinline__ float4 f4add4(const float4 &a, const float4 &b)
+{
+    const float2 lo = __fadd2_rn(make_float2(a.x, a.y), make_float2(b.x, b.y));
+    const float2 hi = __fadd2_rn(make_float2(a.z, a.w), make_float2(b.z, b.w));
+    return make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+__device__ __forceinline__ float4 f4sub(const float4 &a, const float4 &b)
+{
+    float4 r = a;
+    f4fma(r, -1.0f, b);
+    return r;
+}
+// L plus the x part of Eq. 3 at the quad c, from the quads left and right of it.
+// The taps at even distance meet aligned pairs for the output pairs (0, 1) and
+// (2, 3), those at odd distance for the pair (1, 2); outputs 0 and 3 take their
+// odd taps one by one: 22 instructions instead of 32.
+__device__ __forceinline__ float4 lap_x(const float4 &L, const float (&cx)[4], const float4 &lf,
+                                        const float4 &c, const float4 &rt)
+{
+    const float2 l0 = make_float2(lf.x, lf.y), l1 = make_float2(lf.z, lf.w);
+    const float2 c0 = make_float2(c.x, c.y), c1 = make_float2(c.z, c.w);
+    const float2 r0 = make_float2(rt.x, rt.y), r1 = make_float2(rt.z, rt.w);
+    const float2 k1 = make_float2(cx[0], cx[0]), k2 = make_float2(cx[1], cx[1]);
+    const float2 k3 = make_float2(cx[2], cx[2]), k4 = make_float2(cx[3], cx[3]);
+    float2 lo = make_float2(L.x, L.y), hi = make_float2(L.z, L.w);
+    float2 mid = __fmul2_rn(k1, c0);
+    lo = __ffma2_rn(k2, l1, lo);
+    hi = __ffma2_rn(k2, c0, hi);
+    mid = __ffma2_rn(k1, c1, mid);
+    lo = __ffma2_rn(k2, c1, lo);
+    hi = __ffma2_rn(k2, r0, hi);
+    mid = __ffma2_rn(k3, l1, mid);
+    lo = __ffma2_rn(k4, l0, lo);
+    hi = __ffma2_rn(k4, l1, hi);
+    mid = __ffma2_rn(k3, r0, mid);
+    lo = __ffma2_rn(k4, r0, lo);
+    hi = __ffma2_rn(k4, r1, hi);
+    float x = fmaf(cx[0], l1.y, lo.x), w = fmaf(cx[0], c1.x, hi.y);
+    x = fmaf(cx[0], c0.y, x);
+    w = fmaf(cx[0], r0.x, w);
+    x = fmaf(cx[2], l0.y, x);
+    w = fmaf(cx[2], c0.x, w);
+    x = fmaf(cx[2], c1.y, x);
+    w = fmaf(cx[2], r1.x, w);
+    return make_float4(x, __fadd_rn(lo.y, mid.x), __fadd_rn(hi.x, mid.y), w);
+}
 
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 {
@@ -388,6 +468,32 @@ __device__ __forceinline__ void mbar_arrive(uint64_t *bar)
 // (CUDA-graph replays that do not repeat with the buffer parity).
 enum : int { VAR_PLAIN = 0, VAR_SHELL = 1, VAR_FLOW = 2, VAR_PARITY = 3 };
 
+// Position in a ring of N slots of PITCH bytes: the slot's byte offset and the
+// parity of the current pass over the ring.
+template <int N, int PITCH>
+struct RingPos {
+    uint32_t off = 0, ph = 0;
+    __device__ __forceinline__ void next()
+    {
+        off += PITCH;
+        if (off == N * PITCH) {
+            off = 0;
+            ph ^= 1;
+        }
+    }
+    // offset of the slot `back` places behind (back < N)
+    __device__ __forceinline__ uint32_t behind(int back) const
+    {
+        return off >= uint32_t(back) * PITCH ? off - back * PITCH : off + (N - back) * PITCH;
+    }
+    // parity of the last fill of slot s, counting fills up to this position
+    // (a slot that was never filled: a parity that a fresh barrier satisfies)
+    __device__ __forceinline__ uint32_t last_parity(int s) const
+    {
+        return uint32_t(s) * PITCH < off ? ph : ph ^ 1;
+    }
+};
+
 // Per-thread state of one fused-step work unit (a tile x a z-chunk).
 template <class C, class T, int MODE = MODE_FWD, int VAR = VAR_PLAIN>
 struct StepCta {
@@ -399,32 +505,30 @@ struct StepCta {
     // PML receive psi from their PML neighbours
     static constexpr int BAND = MODE == MODE_ADJ ? 1 : 0;
     static constexpr bool SCALED = E::SCALED;
-    static constexpr int TXT = C::TXT, TY = C::TY, NU = Stage<C, T, MODE>::NU, NP = Stage<C, T, MODE>::NP;
-    static constexpr int THREADS = C::THREADS, QN = C::QN, U = C::U, WARPS = C::WARPS;
+    static constexpr int TXT = C::TXT, TY = C::TY, NU = G::NU, NP = G::NP;
+    static constexpr int THREADS = C::THREADS, QN = C::QN, WARPS = C::WARPS;
     static constexpr int BX = C::BX, BY = C::BY, HX = G::HX, SW = G::SW;
     static constexpr int P_TILE = C::P_TILE;
     static constexpr uint64_t WAIT_NS = 2000000000ull;
+    // offsets inside a tile slot: u^{n-1}, m, phi (or the haloed mu box), g^{k-1}, S
+    static constexpr int M_OFF = G::UP_BYTES, PH_OFF = M_OFF + G::F_BYTES;
+    static constexpr int ACC_OFF = PH_OFF + G::PH_BYTES, GS_OFF = ACC_OFF + G::F_BYTES;
 
     const StepArgs *pa;  // the kernel argument, in the constant parameter space
     const CUtensorMap *tm_ucur, *tm_ucur_in, *tm_uprev, *tm_m, *tm_phi, *tm_acc, *tm_gs;
-    unsigned char *su, *sp;  // u ring, (u^{n-1}, m, phi) ring
-    uint64_t *full_u, *empty_u, *full_p, *empty_p;
-    int *lastf_u, *lastf_p, *s_abort;
-    long long base_off;  // element offset of (gi, gj0, k = 0)
-    int tid, lane, x0, y0, z0, z1, n, row0, colu, gi, gj0, prow;
-    bool xy_inner, aborted, store_ok;
+    int tid, x0, y0, z0, z1, n;
+    uint32_t uthr, pthr;  // byte offset of this thread's row-0 quad in a u slot; elements of it in a tile
+    uint32_t toff;        // elements from the tile's corner to it in the padded field
+    bool xy_inner, aborted;
+    // flags of this thread's points, few enough for one register: bits 0-3 its
+    // PML columns, 4 + r a PML row, 8 + 3 r the points of row r's quad inside
+    // the grid (0..4), 16 + r row r's quad holds the source's x and y
+    uint32_t flags;
     int phi_xmask;  // phi blocks holding x-PML columns, when the tile touches only the
                     // x-PML (planes outside the z-PML load only these); 0 otherwise
-    int phoff;      // offset of this thread's row-0 quad in the blocked phi tile
-    int mbox;           // MODE_ADJ: offset of this thread's row-0 quad in the mu box
 
-    // MODE_ADJ: mu^{k+1} at this thread's row-r points one plane below, kept from
-    // plane to plane in shared memory (registers are at their limit)
-    __device__ __forceinline__ float4 *mz_prev(int r) const
-    {
-        return reinterpret_cast<float4 *>(sp + NP * G::P_BYTES) + r * THREADS + tid;
-    }
-    int useq, pseq;  // FLOW: u and (u^{n-1}, m, phi) planes of earlier units of this CTA
+    RingPos<NU, G::U_PITCH> uf;  // front plane k + 4, four slots ahead of plane k (producer: next plane)
+    RingPos<NP, G::P_PITCH> pc;  // (u^{n-1}, m, phi) plane k (producer: next plane)
     void *u_out_v;   // FLOW, PARITY: the output buffer of the current step
     const void *u_cur_v;  // PARITY: u^n of the current step
     float s_cur, s_prev, inv_s_next;  // fp16 scales (1 otherwise)
@@ -433,12 +537,56 @@ struct StepCta {
     // PML terms of the thread's fixed columns i = gi + e and rows j = gj0 + r:
     // eta dt = a d(i)^2, the gradient factor k (d(i+1)^2 - d(i-1)^2), the
     // adjoint's k G(i +- 1) with G(y) = d(y+1)^2 - d(y-1)^2, and PML masks
-    float pex[4], pgx[4], phxp[4], phxm[4];
+    // (x terms as quads over e; nhxm = -k G(i - 1))
+    float4 pex, pgx, phxp, nhxm;
     float pey[TY], pgy[TY], phyp[TY], phym[TY];
-    int pmx, pmy;
     // 1 / (1 + e) and 1 - e of the thread's points in planes outside the z-PML
-    // (e = eta dt depends on x and y only there)
-    float pinv[TY][4], pome[TY][4];
+    // (e = eta dt depends on x and y only there; the adjoint, short of registers,
+    // computes both in every plane)
+    float4 pinv[TY], pome[TY];
+
+    // u slot at ring offset o; tile slot at ring offset o; their barriers
+    __device__ __forceinline__ unsigned char *uslot(uint32_t o) const { return step_smem + o; }
+    __device__ __forceinline__ unsigned char *pslot(uint32_t o) const
+    {
+        return step_smem + NU * G::U_PITCH + o;
+    }
+    __device__ __forceinline__ uint64_t *full_u(uint32_t o) const
+    {
+        return reinterpret_cast<uint64_t *>(uslot(o) + G::U_BYTES);
+    }
+    __device__ __forceinline__ uint64_t *empty_u(uint32_t o) const { return full_u(o) + 1; }
+    __device__ __forceinline__ uint64_t *full_p(uint32_t o) const
+    {
+        return reinterpret_cast<uint64_t *>(pslot(o) + G::P_BYTES);
+    }
+    __device__ __forceinline__ uint64_t *empty_p(uint32_t o) const { return full_p(o) + 1; }
+    __device__ __forceinline__ volatile int *s_abort() const
+    {
+        return reinterpret_cast<volatile int *>(step_smem + G::ABORT_OFF);
+    }
+    __device__ __forceinline__ int tile_quads(int r) const { return (flags >> (8 + 3 * r)) & 7; }
+    // MODE_ADJ: mu^{k+1} at this thread's row-r points one plane below, kept from
+    // plane to plane in shared memory (registers are at their limit)
+    __device__ __forceinline__ float4 *mz_prev(int r) const
+    {
+        return reinterpret_cast<float4 *>(step_smem + G::MZ_OFF) + r * THREADS + tid;
+    }
+
+    // One thread sets the barriers of both rings up (full: the producer's
+    // arrival; empty: one arrival per consumer warp).
+    __device__ __forceinline__ void init_rings(int abort0)
+    {
+        *s_abort() = abort0;
+        for (int i = 0; i < NU; ++i) {
+            mbar_init(full_u(i * G::U_PITCH), 1);
+            mbar_init(empty_u(i * G::U_PITCH), WARPS);
+        }
+        for (int i = 0; i < NP; ++i) {
+            mbar_init(full_p(i * G::P_PITCH), 1);
+            mbar_init(empty_p(i * G::P_PITCH), WARPS);
+        }
+    }
 
     __device__ __forceinline__ void set_maps(const CUtensorMap *ucur, const CUtensorMap *ucur_in,
                                              const CUtensorMap *uprev, const CUtensorMap *m,
@@ -471,23 +619,28 @@ struct StepCta {
     __device__ __forceinline__ void pml_tables()
     {
         const StepArgs &a = *pa;
-        pmx = pmy = 0;
+        const int gi = x0 + 4 * (tid % TXT), gj0 = y0 + TY * (tid / TXT);
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             bool in;
-            pml_axis(a.nx, gi + e, a.ax, a.kx, pex[e], pgx[e], phxp[e], phxm[e], in);
-            pmx |= int(in) << e;
+            float v[4];
+            pml_axis(a.nx, gi + e, a.ax, a.kx, v[0], v[1], v[2], v[3], in);
+            f4set(pex, e, v[0]);
+            f4set(pgx, e, v[1]);
+            f4set(phxp, e, v[2]);
+            f4set(nhxm, e, -v[3]);
+            flags |= uint32_t(in) << e;
         }
 #pragma unroll
         for (int r = 0; r < TY; ++r) {
             bool in;
             pml_axis(a.ny, gj0 + r, a.ay, a.ky, pey[r], pgy[r], phyp[r], phym[r], in);
-            pmy |= int(in) << r;
+            flags |= uint32_t(in) << (4 + r);
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const float exy = __fadd_rn(pex[e], pey[r]);
-                pinv[r][e] = rcp_approx(__fadd_rn(1.0f, exy));
-                pome[r][e] = __fsub_rn(1.0f, exy);
+                const float exy = __fadd_rn(f4get(pex, e), pey[r]);
+                f4set(pinv[r], e, rcp_approx(__fadd_rn(1.0f, exy)));
+                f4set(pome[r], e, __fsub_rn(1.0f, exy));
             }
         }
     }
@@ -497,51 +650,73 @@ struct StepCta {
         return !xy_inner || k < pa->nb + BAND || k >= pa->nb + pa->nz - BAND;
     }
 
-    __device__ __forceinline__ void wait(uint64_t *bar, uint32_t parity)
+    // Bounded wait of the calling thread: false (and the CTA's abort flag set)
+    // after WAIT_NS, or as soon as another thread of the CTA has given up.
+    __device__ __forceinline__ bool spin(uint64_t *bar, uint32_t parity)
     {
-        if (!mbar_wait_bounded(bar, parity, WAIT_NS)) {
-            *reinterpret_cast<volatile int *>(s_abort) = 1;
-            atomicOr(pa->err, DEV_ERR_TIMEOUT);
+        uint64_t t0 = 0;
+        for (;;) {
+#pragma unroll 1
+            for (int i = 0; i < 32; ++i)  // the timer read is slow: between batches of polls
+                if (mbar_try_wait(bar, parity)) return true;
+            if (*s_abort()) return false;
+            const uint64_t t = global_timer_ns();
+            if (t0 == 0) t0 = t;
+            if (t - t0 > WAIT_NS) {
+                *s_abort() = 1;
+                atomicOr(pa->err, DEV_ERR_TIMEOUT);
+                return false;
+            }
         }
     }
 
-    __device__ __forceinline__ const T *ustage(int s) const
+    // ... of one thread; sets aborted when it gives up.
+    __device__ __forceinline__ void wait(uint64_t *bar, uint32_t parity)
     {
-        return reinterpret_cast<const T *>(su + s * G::U_BYTES);
+        if (!mbar_try_wait(bar, parity) && !spin(bar, parity)) aborted = true;
     }
 
-    // Planes outside the chunk feed only the z-queue: no x-y halo needed.
+    // ... of a whole warp; aborted stays uniform over it.
+    __device__ __forceinline__ void wait_warp(uint64_t *bar, uint32_t parity)
+    {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return;
+        const bool ok = spin(bar, parity);
+        if (!__all_sync(0xffffffffu, ok)) aborted = true;
+    }
+
+    // Planes outside the chunk feed only the z-queue: they need no x-y halo (but
+    // land at their place in a full slot, x margin included).
     __device__ __forceinline__ bool front_only(int p) const { return p < z0 || p >= z1; }
 
-    // Offset, inside a u stage holding plane p, of this thread's row-r quad.
-    __device__ __forceinline__ int own_off(int p, int r) const
+    // This thread's row-r quad in the u slot at ring offset o.
+    __device__ __forceinline__ const T *own_ptr(uint32_t o, int r) const
     {
-        return front_only(p) ? prow + r * BX : (row0 + r) * SW + colu;
+        return reinterpret_cast<const T *>(uslot(o) + uthr) + r * SW;
     }
 
     __device__ __forceinline__ void issue_u(int p)
     {
-        const int rel = p - z0 + 4 + (FLOW ? useq : 0);
-        const int s = rel % NU, f = rel / NU;
-        if (f > 0) wait(empty_u + s, (f - 1) & 1);  // previous plane of the slot released
-        lastf_u[s] = f;
+        const uint32_t o = uf.off;
+        wait(empty_u(o), uf.ph ^ 1);  // previous plane of the slot released (true on the first pass)
+        if (aborted) return;
+        uf.next();
         if (front_only(p)) {
-            mbar_arrive_expect_tx(full_u + s, P_TILE * (int)sizeof(T));
+            mbar_arrive_expect_tx(full_u(o), SW * BY * (int)sizeof(T));
             // a neighbouring z-chunk's plane: kept in L2 for that chunk's own read
-            tma_load_3d_hint(su + s * G::U_BYTES, tm_ucur_in, full_u + s, x0, y0, p,
+            tma_load_3d_hint(uslot(o) + R * SW * (int)sizeof(T), tm_ucur_in, full_u(o), x0 - HX, y0, p,
                              policy_evict_last());
         } else {
-            mbar_arrive_expect_tx(full_u + s, SW * C::SH * (int)sizeof(T));
-            tma_load_3d(su + s * G::U_BYTES, tm_ucur, full_u + s, x0 - HX, y0 - R, p);
+            mbar_arrive_expect_tx(full_u(o), SW * C::SH * (int)sizeof(T));
+            tma_load_3d(uslot(o), tm_ucur, full_u(o), x0 - HX, y0 - R, p);
         }
     }
 
     __device__ __forceinline__ void issue_p(int k)
     {
-        const int rel = k - z0 + (FLOW ? pseq : 0);
-        const int s = rel % NP, f = rel / NP;
-        if (f > 0) wait(empty_p + s, (f - 1) & 1);
-        lastf_p[s] = f;
+        const uint32_t o = pc.off;
+        wait(empty_p(o), pc.ph ^ 1);
+        if (aborted) return;
+        pc.next();
         const bool pml = plane_pml(k);
         const bool zpml = k < pa->nb || k >= pa->nb + pa->nz;
         const int phmask = !pml ? 0 : (phi_xmask && !zpml) ? phi_xmask : (1 << C::PHI_NB) - 1;
@@ -549,24 +724,24 @@ struct StepCta {
         constexpr int PHB_BYTES = C::PHI_BW * C::BY * 4;
         const int ph_bytes = MODE == MODE_ADJ ? (pml ? G::MBW * G::MBH * 4 : 0)
                                               : __popc(phmask) * PHB_BYTES;
-        mbar_arrive_expect_tx(full_p + s, P_TILE * (int)sizeof(T) + ntiles * G::F_BYTES + ph_bytes);
-        unsigned char *d = sp + s * G::P_BYTES;
+        uint64_t *full = full_p(o);
+        mbar_arrive_expect_tx(full, P_TILE * (int)sizeof(T) + ntiles * G::F_BYTES + ph_bytes);
+        unsigned char *d = pslot(o);
         // No evict-first hint: u^{n-1} and phi are overwritten in place (u^{n+1},
         // phi^{n+1}) a few planes later, and marking their lines first-to-go cost
         // 8% of the step at 512^3 (118 MB more DRAM read per launch).
-        tma_load_3d(d, tm_uprev, full_p + s, x0, y0, k);
-        tma_load_3d(d + G::UP_BYTES, tm_m, full_p + s, x0, y0, k);
+        tma_load_3d(d, tm_uprev, full, x0, y0, k);
+        tma_load_3d(d + M_OFF, tm_m, full, x0, y0, k);
         if constexpr (MODE == MODE_ADJ) {
             // mu^{k+1} with its x-y halo; g^{k-1} of the recomputation; partial sum S
-            if (pml) tma_load_3d(d + G::UP_BYTES + G::F_BYTES, tm_phi, full_p + s, x0 - 4, y0 - 1, k);
-            tma_load_3d(d + G::UP_BYTES + G::F_BYTES + G::PH_BYTES, tm_acc, full_p + s, x0, y0, k);
-            tma_load_3d(d + G::UP_BYTES + 2 * G::F_BYTES + G::PH_BYTES, tm_gs, full_p + s, x0, y0, k);
+            if (pml) tma_load_3d(d + PH_OFF, tm_phi, full, x0 - 4, y0 - 1, k);
+            tma_load_3d(d + ACC_OFF, tm_acc, full, x0, y0, k);
+            tma_load_3d(d + GS_OFF, tm_gs, full, x0, y0, k);
         } else {
 #pragma unroll
             for (int b = 0; b < C::PHI_NB; ++b)
                 if ((phmask >> b) & 1)
-                    tma_load_3d(d + G::UP_BYTES + G::F_BYTES + b * PHB_BYTES, tm_phi, full_p + s,
-                                x0 + b * C::PHI_BW, y0, k);
+                    tma_load_3d(d + PH_OFF + b * PHB_BYTES, tm_phi, full, x0 + b * C::PHI_BW, y0, k);
         }
     }
 
@@ -589,66 +764,60 @@ struct StepCta {
             const bool do_u = nu < z1 + 4 && (np >= z1 || nu - z0 - 4 <= np - z0);
             if (do_u) issue_u(nu++);
             else issue_p(np++);
-            aborted = *reinterpret_cast<volatile int *>(s_abort) != 0;
         }
     }
 
     __device__ __forceinline__ void drain()
     {
         for (int s = 0; s < NU; ++s)
-            if (lastf_u[s] >= 0) mbar_wait_bounded(full_u + s, lastf_u[s] & 1, WAIT_NS);
+            mbar_wait_bounded(full_u(s * G::U_PITCH), uf.last_parity(s), WAIT_NS);
         for (int s = 0; s < NP; ++s)
-            if (lastf_p[s] >= 0) mbar_wait_bounded(full_p + s, lastf_p[s] & 1, WAIT_NS);
+            mbar_wait_bounded(full_p(s * G::P_PITCH), pc.last_parity(s), WAIT_NS);
     }
 
-    // One z-plane: iteration it (plane k = z0 + it).  The queue holds planes
-    // k-4 .. k+3 at q[O .. O+7]; the front plane k+4 is loaded into q[O+8].
+    // One z-plane k.  The queue holds planes k-4 .. k+3 at q[0 .. 7]; the front
+    // plane k+4 is loaded into q[8].
     // Queue values are the stored (scaled) values; true u = stored * s_cur.
     // KIND: PLANE_INTERIOR (no PML point in the tile's plane), PLANE_XY (PML
     // path, plane outside the z-PML: e from the thread's tables), PLANE_Z (a
     // z-PML plane).
-    template <int O, int KIND>
-    __device__ __forceinline__ void plane(float4 (&q)[TY][QN], int it)
+    template <int KIND>
+    __device__ __forceinline__ void plane(float4 (&q)[TY][QN], int k)
     {
         constexpr bool PML = KIND != PLANE_INTERIOR;
         constexpr bool ZP = KIND == PLANE_Z;
         const StepArgs &a = *pa;
-        const int k = z0 + it;
-        const int relf = it + 8 + (FLOW ? useq : 0);
-        const int sf = relf % NU;
-        wait(full_u + sf, (relf / NU) & 1);
+        {
+            const bool fu = mbar_try_wait(full_u(uf.off), uf.ph), fp = mbar_try_wait(full_p(pc.off), pc.ph);
+            if (!__all_sync(0xffffffffu, fu && fp)) {
+#pragma unroll 1
+                for (int w = 0; w < 2; ++w)
+                    wait_warp(w ? full_p(pc.off) : full_u(uf.off), w ? pc.ph : uf.ph);
+            }
+        }
 #pragma unroll
-        for (int r = 0; r < TY; ++r) q[r][O + 8] = E::ld(ustage(sf) + own_off(k + 4, r));
-        const int itp = it + (FLOW ? pseq : 0);
-        const int sq = itp % NP;
-        wait(full_p + sq, (itp / NP) & 1);
-        const int sc = (it + 4 + (FLOW ? useq : 0)) % NU;
-        const T *cu = ustage(sc);
-        const unsigned char *pu = sp + sq * G::P_BYTES;
-        const T *pup = reinterpret_cast<const T *>(pu);
-        const float *pm = reinterpret_cast<const float *>(pu + G::UP_BYTES);
-        const float *pph = reinterpret_cast<const float *>(pu + G::UP_BYTES + G::F_BYTES);
-        const float *pg = reinterpret_cast<const float *>(pu + G::UP_BYTES + G::F_BYTES + G::PH_BYTES);
-        const float *pgs =
-            reinterpret_cast<const float *>(pu + G::UP_BYTES + 2 * G::F_BYTES + G::PH_BYTES);
+        for (int r = 0; r < TY; ++r) q[r][8] = E::ld(own_ptr(uf.off, r));
+        const unsigned char *pu = pslot(pc.off);
+        const uint32_t uc = uf.behind(4);  // plane k
+        const T *cu = own_ptr(uc, 0);
 
         // 25-point Laplacian (Eq. 3): centre and z part from the queue
         float4 L[TY], gy[TY];
 #pragma unroll
         for (int r = 0; r < TY; ++r) {
-            L[r] = f4mul(a.c0, q[r][O + 4]);
+            L[r] = f4mul(a.c0, q[r][4]);
 #pragma unroll
             for (int m = 1; m <= R; ++m) {
-                f4fma(L[r], a.cz[m - 1], q[r][O + 4 - m]);
-                f4fma(L[r], a.cz[m - 1], q[r][O + 4 + m]);
+                f4fma(L[r], a.cz[m - 1], q[r][4 - m]);
+                f4fma(L[r], a.cz[m - 1], q[r][4 + m]);
             }
         }
         // y part: rows -4 .. TY+3 around the thread's first row
 #pragma unroll
         for (int d = -R; d < TY + R; ++d) {
             float4 v;
-            if (d >= 0 && d < TY) v = q[d][O + 4];
-            else v = E::ld(cu + (row0 + d) * SW + colu);
+            if (d >= 0 && d < TY) v = q[d][4];
+            else v = E::ld(cu + d * SW);
 #pragma unroll
             for (int r = 0; r < TY; ++r) {
                 const int m = d > r ? d - r : r - d;
@@ -661,31 +830,22 @@ struct StepCta {
         float ez = 0.f, gzk = 0.f, hzp = 0.f, hzm = 0.f;
         bool zin = false;
         if (PML) pml_axis(a.nz, k, a.az, a.kz, ez, gzk, hzp, hzm, zin);
-        const long long off0 = base_off + (long long)k * a.sxy;
+        // the tile's corner in the padded fields
+        const long long off0 = a.origin + (long long)k * a.sxy + (long long)y0 * a.sx + x0;
         // random bits of this thread's stores in this plane (16-bit storage)
         uint32_t rnd = 0;
-        if constexpr (sizeof(T) == 2) rnd = hash_bits((uint32_t)off0, (uint32_t)n);
+        if constexpr (sizeof(T) == 2) rnd = hash_bits((uint32_t)off0 + toff, (uint32_t)n);
 #pragma unroll
         for (int r = 0; r < TY; ++r) {
-            const T *rowp = cu + (row0 + r) * SW + colu;
-            float4 c = q[r][O + 4];
+            const T *rowp = cu + r * SW;
+            const uint32_t ro = toff + r * (uint32_t)a.sx;  // this row's quad from the tile's corner
+            float4 c = q[r][4];
             const float4 lf = E::ld(rowp - 4), rt = E::ld(rowp + 4);
-            const float w[12] = {lf.x, lf.y, lf.z, lf.w, c.x, c.y, c.z, c.w,
-                                 rt.x, rt.y, rt.z, rt.w};
-            float4 Lr = L[r];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                float sacc = f4get(Lr, e);
-#pragma unroll
-                for (int m = 1; m <= R; ++m) {
-                    sacc = fmaf(a.cx[m - 1], w[4 + e - m], sacc);
-                    sacc = fmaf(a.cx[m - 1], w[4 + e + m], sacc);
-                }
-                f4set(Lr, e, sacc);
-            }
-            const int pr = prow + r * BX;
-            float4 up = E::ld(pup + pr);
-            const float4 mm = lds128(pm + pr);
+            const float4 cs = c;  // stored values
+            float4 Lr = lap_x(L[r], a.cx, lf, c, rt);
+            const uint32_t pr = pthr + r * BX;
+            float4 up = E::ld(reinterpret_cast<const T *>(pu) + pr);
+            const float4 mm = lds128(reinterpret_cast<const float *>(pu + M_OFF) + pr);
             if constexpr (SCALED) {  // stored values -> true values
                 Lr = f4mul(s_cur, Lr);
                 c = f4mul(s_cur, c);
@@ -693,97 +853,83 @@ struct StepCta {
             }
             float4 un;  // MODE_DIFF: d^{n+1} until the source is added
             if constexpr (MODE == MODE_DIFF) {  // up = d^n: d^{n+1} = d^n + m L u^n
-                un.x = fmaf(mm.x, Lr.x, up.x);
-                un.y = fmaf(mm.y, Lr.y, up.y);
-                un.z = fmaf(mm.z, Lr.z, up.z);
-                un.w = fmaf(mm.w, Lr.w, up.w);
+                un = f4fma4(mm, Lr, up);
             } else {
-                un.x = fmaf(mm.x, Lr.x, fmaf(2.0f, c.x, -up.x));
-                un.y = fmaf(mm.y, Lr.y, fmaf(2.0f, c.y, -up.y));
-                un.z = fmaf(mm.z, Lr.z, fmaf(2.0f, c.z, -up.z));
-                un.w = fmaf(mm.w, Lr.w, fmaf(2.0f, c.w, -up.w));
+                un = f4fma4(mm, Lr, make_float4(fmaf(2.0f, c.x, -up.x), fmaf(2.0f, c.y, -up.y),
+                                                fmaf(2.0f, c.z, -up.z), fmaf(2.0f, c.w, -up.w)));
             }
-            const int j = gj0 + r;
             float4 phn = make_float4(0.f, 0.f, 0.f, 0.f);
-            bool any_pml = false;
-            int ptmask = 0;
             float4 ph = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (PML) {
-                if constexpr (MODE == MODE_ADJ) ph = lds128(pph + mbox + r * G::MBW);
-                else ph = lds128(pph + phoff + r * C::PHI_BW);
-                phn = ph;
-                const float eyz = ZP ? __fadd_rn(pey[r], ez) : 0.0f;
-                const float gyk = pgy[r];
-                // bit e: point e of this row is a PML point
-                const int rowmask = (ZP || zin || ((pmy >> r) & 1)) ? 0xF : pmx;
-                const float4 zp = q[r][O + 5], zm = q[r][O + 3];
-                // adjoint: psi = sum_a k_a [G_a mu](x + e_a) - [G_a mu](x - e_a) from the six
-                // neighbours of mu^{k+1} (zero outside the PML and in the halo): x and y
-                // from the haloed box, -z kept from the plane below, +z from global memory
-                float4 myp = make_float4(0.f, 0.f, 0.f, 0.f), mym = myp, mzp = myp, mzm = myp;
-                float mxl = 0.f, mxr = 0.f;
-                if constexpr (MODE == MODE_ADJ) {
-                    const float *mb = pph + mbox + r * G::MBW;
-                    myp = lds128(mb + G::MBW);
-                    mym = lds128(mb - G::MBW);
-                    mxl = mb[-1];
-                    mxr = mb[4];
-                    mzm = *mz_prev(r);
-                    if (store_ok && j < a.Ny) mzp = ldg128(a.mu_in + off0 + (long long)r * a.sx + a.sxy);
-                    *mz_prev(r) = ph;
+            int rowmask = 0;  // bit e: point e of this row is a PML point
+            if constexpr (PML) {
+                const float *pph = reinterpret_cast<const float *>(pu + PH_OFF);
+                rowmask = (ZP || zin || ((flags >> (4 + r)) & 1)) ? 0xF : flags & 0xF;
+                // 1 / (1 + e), 1 - e
+                float4 inv = pinv[r], ome = pome[r];
+                if constexpr (ZP || MODE == MODE_ADJ) {
+                    const float eyz = ZP ? __fadd_rn(pey[r], ez) : pey[r];
+                    const float4 ed = f4add4(make_float4(eyz, eyz, eyz, eyz), pex);
+                    const float4 one = make_float4(1.0f, 1.0f, 1.0f, 1.0f);
+                    const float4 oe = f4add4(one, ed);
+                    ome = f4sub(one, ed);
+                    inv = make_float4(rcp_approx(oe.x), rcp_approx(oe.y), rcp_approx(oe.z),
+                                      rcp_approx(oe.w));
                 }
-                const float mux[6] = {mxl, ph.x, ph.y, ph.z, ph.w, mxr};
+                float4 rhs;  // phi^n (forward) or psi (adjoint)
+                if constexpr (MODE == MODE_ADJ) {
+                    // psi = sum_a k_a [G_a mu](x + e_a) - [G_a mu](x - e_a) from the six
+                    // neighbours of mu^{k+1} (zero outside the PML and in the halo): x and y
+                    // from the haloed box, -z kept from the plane below, +z from global memory
+                    const float *mb = pph + mu_off() + r * G::MBW;
+                    ph = lds128(mb);
+                    const float4 myp = lds128(mb + G::MBW), mym = lds128(mb - G::MBW);
+                    const float4 mzm = *mz_prev(r);
+                    float4 mzp = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (tile_quads(r)) mzp = ldg128(a.mu_in + (off0 + a.sxy) + ro);
+                    *mz_prev(r) = ph;
+                    rhs = f4mul4(nhxm, make_float4(mb[-1], ph.x, ph.y, ph.z));
+                    rhs = f4fma4(phxp, make_float4(ph.y, ph.z, ph.w, mb[4]), rhs);
+                    f4fma(rhs, phyp[r], myp);
+                    f4fma(rhs, -phym[r], mym);
+                    f4fma(rhs, hzp, mzp);
+                    f4fma(rhs, -hzm, mzm);
+                } else {
+                    ph = lds128(pph + phi_off() + r * C::PHI_BW);
+                    rhs = ph;
+                }
+                const float4 lr = f4add4(Lr, rhs);
+                float4 upml;
+                if constexpr (MODE == MODE_DIFF) {
+                    // d^{n+1} = u^{n+1} - c with u^{n-1} = c - d^n:
+                    //   [(1 - e) d^n + m lr - e^2 c] / (1 + e)
+                    const float4 ed = f4sub(make_float4(1.0f, 1.0f, 1.0f, 1.0f), ome);
+                    const float4 e2c = f4mul4(f4mul4(ed, ed), c);
+                    upml = f4mul4(inv, f4fma4(mm, lr, f4fma4(ome, up, f4mul(-1.0f, e2c))));
+                } else {
+                    // [(2 - e^2) c - (1 - e) u^{n-1} + m lr] / (1 + e)
+                    //   = (1 - e) c + [c - (1 - e) u^{n-1} + m lr] / (1 + e)
+                    upml = f4fma4(inv, f4fma4(mm, lr, f4fma4(ome, f4mul(-1.0f, up), c)), f4mul4(ome, c));
+                }
+                if constexpr (MODE == MODE_ADJ) {
+                    // psi also reaches the inner points next to the PML;
+                    // mu^k = (mu^{k+1} + w^{k+1}) / (1 + e) on the PML
+                    un = f4fma4(mm, lr, make_float4(fmaf(2.0f, c.x, -up.x), fmaf(2.0f, c.y, -up.y),
+                                                    fmaf(2.0f, c.z, -up.z), fmaf(2.0f, c.w, -up.w)));
+                    phn = f4mul4(f4add4(ph, c), inv);
+                } else {
+                    // dt grad(eta) . grad(u)
+                    float4 gd = f4mul(gzk, f4sub(q[r][5], q[r][3]));
+                    f4fma(gd, pgy[r], gy[r]);
+                    gd = f4fma4(pgx, make_float4(__fsub_rn(cs.y, lf.w), __fsub_rn(cs.z, cs.x),
+                                                 __fsub_rn(cs.w, cs.y), __fsub_rn(rt.x, cs.z)), gd);
+                    if constexpr (SCALED) gd = f4mul(s_cur, gd);
+                    phn = f4mul4(f4sub(ph, gd), inv);
+                }
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const bool pt = (rowmask >> e) & 1;
-                    any_pml |= pt;
-                    float Gd = fmaf(pgx[e], __fsub_rn(w[5 + e], w[3 + e]),
-                                    fmaf(gyk, f4get(gy[r], e),
-                                         __fmul_rn(gzk, __fsub_rn(f4get(zp, e), f4get(zm, e)))));
-                    if constexpr (SCALED) Gd = __fmul_rn(Gd, s_cur);
-                    float inv, ome;  // 1 / (1 + e), 1 - e
-                    if constexpr (ZP) {
-                        const float edt = __fadd_rn(pex[e], eyz);
-                        inv = rcp_approx(__fadd_rn(1.0f, edt));
-                        ome = __fsub_rn(1.0f, edt);
-                    } else {
-                        inv = pinv[r][e];
-                        ome = pome[r][e];
-                    }
-                    const float cc = f4get(c, e), pe = f4get(ph, e);
-                    float rhs = pe;  // phi^n (forward) or psi (adjoint)
-                    if constexpr (MODE == MODE_ADJ) {
-                        rhs = fmaf(phxp[e], mux[e + 2], __fmul_rn(-phxm[e], mux[e]));
-                        rhs = fmaf(phyp[r], f4get(myp, e), rhs);
-                        rhs = fmaf(-phym[r], f4get(mym, e), rhs);
-                        rhs = fmaf(hzp, f4get(mzp, e), rhs);
-                        rhs = fmaf(-hzm, f4get(mzm, e), rhs);
-                    }
-                    const float lr = __fadd_rn(f4get(Lr, e), rhs);
-                    float upml;
-                    if constexpr (MODE == MODE_DIFF) {
-                        // d^{n+1} = u^{n+1} - c with u^{n-1} = c - d^n:
-                        //   [(1 - e) d^n + m lr - e^2 c] / (1 + e)
-                        const float ed = __fsub_rn(1.0f, ome);
-                        upml = __fmul_rn(inv, fmaf(f4get(mm, e), lr,
-                                                   fmaf(ome, f4get(up, e), -__fmul_rn(__fmul_rn(ed, ed), cc))));
-                    } else {
-                        // [(2 - e^2) c - (1 - e) u^{n-1} + m lr] / (1 + e)
-                        //   = (1 - e) c + [c - (1 - e) u^{n-1} + m lr] / (1 + e)
-                        upml = fmaf(inv, fmaf(f4get(mm, e), lr, fmaf(-ome, f4get(up, e), cc)),
-                                    __fmul_rn(ome, cc));
-                    }
-                    const float ppml = __fmul_rn(__fsub_rn(pe, Gd), inv);
-                    ptmask |= int(pt) << e;
-                    if constexpr (MODE == MODE_ADJ) {
-                        // psi also reaches the inner points next to the PML;
-                        // mu^k = (mu^{k+1} + w^{k+1}) / (1 + e) on the PML
-                        f4set(un, e, pt ? upml : fmaf(f4get(mm, e), lr, fmaf(2.0f, cc, -f4get(up, e))));
-                        if (pt) f4set(phn, e, __fmul_rn(__fadd_rn(pe, cc), inv));
-                    } else if (pt) {
-                        f4set(un, e, upml);
-                        f4set(phn, e, ppml);
-                    }
+                    f4set(un, e, pt ? f4get(upml, e) : f4get(un, e));
+                    f4set(phn, e, pt ? f4get(phn, e) : f4get(ph, e));
                 }
             }
             if constexpr (MODE == MODE_ADJ && !PML) *mz_prev(r) = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -791,14 +937,14 @@ struct StepCta {
             if constexpr (MODE == MODE_FWD_ACC) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
-                    if ((ptmask >> e) & 1) f4set(acc4, e, f4get(acc4, e) + f4get(ph, e));
+                    if ((rowmask >> e) & 1) f4set(acc4, e, __fadd_rn(f4get(acc4, e), f4get(ph, e)));
             }
             // point source (Eq. 2 right-hand side), added by the owning thread
-            if (MODE != MODE_ADJ && k == a.sk && j == a.sj && a.si >= gi && a.si < gi + 4) {
-                const int e = a.si - gi;
+            if (MODE != MODE_ADJ && k == a.sk && ((flags >> (16 + r)) & 1)) {
+                const int e = a.si & 3;  // tiles start at multiples of 4
                 const float f = a.wavelet[n] * a.inv_vol;
                 f4set(un, e, fmaf(f4get(mm, e), f, f4get(un, e)));
-                if constexpr (MODE == MODE_FWD_ACC) f4set(acc4, e, f4get(acc4, e) + f);
+                if constexpr (MODE == MODE_FWD_ACC) f4set(acc4, e, __fadd_rn(f4get(acc4, e), f));
             }
             float4 dn;  // MODE_DIFF: d^{n+1}; u^{n+1} = u^n + d^{n+1}
             if constexpr (MODE == MODE_DIFF) {
@@ -808,10 +954,12 @@ struct StepCta {
             }
             // shell launches leave the box to the two-step kernel (its x bounds
             // are multiples of 4: a quad is wholly inside or outside)
+            const int gi = x0 + 4 * (tid % TXT), j = y0 + TY * (tid / TXT) + r;
             const bool boxed = SHELL && gi >= a.bx0 && gi < a.bx1 && j >= a.by0 && j < a.by1 &&
                                k >= a.bz0 && k < a.bz1;
-            if (store_ok && j < a.Ny && !boxed) {
-                const long long off = off0 + (long long)r * a.sx;
+            const int nst = tile_quads(r);
+            if (nst && !boxed) {
+                const long long off = off0 + ro;
                 if constexpr (SCALED) {
                     vmax = fmaxf(vmax, fmaxf(fmaxf(fabsf(un.x), fabsf(un.y)),
                                              fmaxf(fabsf(un.z), fabsf(un.w))));
@@ -823,49 +971,47 @@ struct StepCta {
                     }
                 }
                 T *uo = static_cast<T *>(OUTV ? u_out_v : a.u_out) + off;
-                const bool wphi = PML && any_pml;  // phi^{n+1}, or mu^k in the adjoint
+                const bool wphi = PML && rowmask;  // phi^{n+1}, or mu^k in the adjoint
                 // MODE_DIFF: d^{n+1} rounded with its own random word (an odd
                 // multiple of u's, so uniform and distinct)
                 T *dio = nullptr;
                 if constexpr (MODE == MODE_DIFF) dio = static_cast<T *>(a.d_io) + off;
                 const uint32_t rnd_d = rnd * 0x2C1B3C6Du;
-                if (gi + 3 < a.Nx) {
-                    E::st(uo, un, rnd);
-                    if constexpr (MODE == MODE_DIFF) E::st(dio, dn, rnd_d);
-                    if (wphi) stg128(a.phi + off, phn);
-                    if constexpr (MODE == MODE_FWD_ACC) stg128(a.acc_out + off, acc4);
-                } else {
-                    for (int e = 0; e < 4 && gi + e < a.Nx; ++e) {
-                        E::put(uo + e, f4get(un, e), hash_bits(rnd, (uint32_t)e));
-                        if constexpr (MODE == MODE_DIFF)
-                            E::put(dio + e, f4get(dn, e), hash_bits(rnd_d, (uint32_t)e));
-                        if (wphi) a.phi[off + e] = f4get(phn, e);
-                        if constexpr (MODE == MODE_FWD_ACC) a.acc_out[off + e] = f4get(acc4, e);
-                    }
-                }
-                if constexpr (sizeof(T) == 2) rnd = next_bits(rnd);  // the next row's word
+                float4 s4 = make_float4(0.f, 0.f, 0.f, 0.f);
                 if constexpr (MODE == MODE_ADJ) {
                     // S += w^k g^{k-1} (dJ/dm = sum_k w^k g^{k-1} / m; S is folded
                     // into the fp64 sum every few steps)
-                    const float4 gk = lds128(pg + pr);
-                    float4 s4 = lds128(pgs + pr);
+                    const float4 gk = lds128(reinterpret_cast<const float *>(pu + ACC_OFF) + pr);
+                    s4 = lds128(reinterpret_cast<const float *>(pu + GS_OFF) + pr);
                     s4.x = fmaf(un.x, gk.x, s4.x);
                     s4.y = fmaf(un.y, gk.y, s4.y);
                     s4.z = fmaf(un.z, gk.z, s4.z);
                     s4.w = fmaf(un.w, gk.w, s4.w);
-                    if (gi + 3 < a.Nx) stg128(a.gsum + off, s4);
-                    else
-                        for (int e = 0; e < 4 && gi + e < a.Nx; ++e) a.gsum[off + e] = f4get(s4, e);
                 }
+                if (nst == 4) {
+                    E::template st<true>(uo, un, rnd, 4);
+                    if constexpr (MODE == MODE_DIFF) E::template st<true>(dio, dn, rnd_d, 4);
+                    if (wphi) stg128(a.phi + off, phn);
+                    if constexpr (MODE == MODE_FWD_ACC) stg128(a.acc_out + off, acc4);
+                    if constexpr (MODE == MODE_ADJ) stg128(a.gsum + off, s4);
+                } else {
+                    E::template st<false>(uo, un, rnd, nst);
+                    if constexpr (MODE == MODE_DIFF) E::template st<false>(dio, dn, rnd_d, nst);
+                    if (wphi) st_part(a.phi + off, phn, nst);
+                    if constexpr (MODE == MODE_FWD_ACC) st_part(a.acc_out + off, acc4, nst);
+                    if constexpr (MODE == MODE_ADJ) st_part(a.gsum + off, s4, nst);
+                }
+                if constexpr (sizeof(T) == 2) rnd = next_bits(rnd);  // the next row's word
             }
         }
-        // release the current u plane and this p slot
+        // release the current u plane and this tile slot
         __syncwarp();
-        if (lane == 0) {
-            mbar_arrive(empty_u + sc);
-            mbar_arrive(empty_p + sq);
+        if ((tid & 31) == 0) {
+            mbar_arrive(empty_u(uc));
+            mbar_arrive(empty_p(pc.off));
         }
-        aborted = *reinterpret_cast<volatile int *>(s_abort) != 0;
+        uf.next();
+        pc.next();
     }
 
     // Tile-level geometry of the unit (x0, y0, z0, z1 set): whether the tile
@@ -891,16 +1037,28 @@ struct StepCta {
     {
         const StepArgs &a = *pa;
         const int txi = tid % C::TXT, tyi = tid / C::TXT;
-        row0 = R + TY * tyi;
-        colu = G::HX + 4 * txi;
-        gi = x0 + 4 * txi;
-        gj0 = y0 + TY * tyi;
-        prow = (TY * tyi) * BX + 4 * txi;
-        phoff = (4 * txi / C::PHI_BW) * C::PHI_BW * BY + (TY * tyi) * C::PHI_BW + (4 * txi) % C::PHI_BW;
-        store_ok = gi < a.Nx;
-        base_off = a.origin + (long long)gj0 * a.sx + gi;
+        const int gi = x0 + 4 * txi, gj0 = y0 + TY * tyi;
+        uthr = ((R + TY * tyi) * SW + HX + 4 * txi) * (int)sizeof(T);
+        pthr = (TY * tyi) * BX + 4 * txi;
+        toff = (uint32_t)(TY * tyi) * (uint32_t)a.sx + 4 * txi;
+        flags = 0;
+#pragma unroll
+        for (int r = 0; r < TY; ++r) {
+            if (gj0 + r < a.Ny) flags |= uint32_t(min(max(a.Nx - gi, 0), 4)) << (8 + 3 * r);
+            if (gj0 + r == a.sj && a.si >= gi && a.si < gi + 4) flags |= 1u << (16 + r);
+        }
         pml_tables();
-        if constexpr (MODE == MODE_ADJ) mbox = (1 + TY * tyi) * G::MBW + 4 + 4 * txi;
+    }
+    // MODE_ADJ: this thread's row-0 quad in the haloed mu box.
+    __device__ __forceinline__ int mu_off() const
+    {
+        return (1 + TY * (tid / TXT)) * G::MBW + 4 + 4 * (tid % TXT);
+    }
+    // This thread's row-0 quad in the blocked phi tile.
+    __device__ __forceinline__ int phi_off() const
+    {
+        const int c = 4 * (tid % TXT);
+        return (c / C::PHI_BW) * C::PHI_BW * BY + (TY * (tid / TXT)) * C::PHI_BW + c % C::PHI_BW;
     }
 
     // Prime the register queue with planes z0-4 .. z0+3 and run the unit's
@@ -911,74 +1069,71 @@ struct StepCta {
     __device__ __forceinline__ void consume_unit(float4 (&q)[TY][QN])
     {
         const StepArgs &a = *pa;
-        const int nit = z1 - z0;
-        const int u0 = FLOW ? useq : 0;
         if constexpr (MODE == MODE_ADJ) {  // mu^{k+1} one plane below the unit
+            const long long off0 = a.origin + (long long)(z0 - 1) * a.sxy + (long long)y0 * a.sx + x0;
 #pragma unroll
             for (int r = 0; r < TY; ++r)
-                *mz_prev(r) = store_ok && gj0 + r < a.Ny
-                                 ? ldg128(a.mu_in + base_off + (long long)(z0 - 1) * a.sxy +
-                                          (long long)r * a.sx)
-                                 : make_float4(0.f, 0.f, 0.f, 0.f);
+                *mz_prev(r) = tile_quads(r) ? ldg128(a.mu_in + off0 + toff + r * (uint32_t)a.sx)
+                                            : make_float4(0.f, 0.f, 0.f, 0.f);
         }
 #pragma unroll
-        for (int s = 0; s < 8; ++s) {
-            wait(full_u + (u0 + s) % NU, ((u0 + s) / NU) & 1);
+        for (int h = 0; h < 2; ++h) {
+            auto ahead = uf;
+#pragma unroll 1
+            for (int s = 0; s < 4; ++s) {
+                wait_warp(full_u(ahead.off), ahead.ph);
+                ahead.next();
+            }
 #pragma unroll
-            for (int r = 0; r < TY; ++r) q[r][s] = E::ld(ustage((u0 + s) % NU) + own_off(z0 - 4 + s, r));
-        }
-        // planes z0-4 .. z0-1 are not needed again
-        __syncwarp();
-        if (lane == 0)
-            for (int s = 0; s < 4; ++s) mbar_arrive(empty_u + (u0 + s) % NU);
-        aborted = *reinterpret_cast<volatile int *>(s_abort) != 0;
-        const int zlo = min(max(a.nb - z0, 0), nit);
-        const int zhi = min(max(a.nb + a.nz - z0, zlo), nit);
-        segment<PLANE_Z>(q, 0, zlo);
-        if (!xy_inner) {
-            segment<PLANE_XY>(q, zlo, zhi);
-        } else {
-            const int b0 = min(max(a.nb + BAND - z0, zlo), zhi);
-            const int b1 = min(max(a.nb + a.nz - BAND - z0, b0), zhi);
-            segment<PLANE_XY>(q, zlo, b0);
-            segment<PLANE_INTERIOR>(q, b0, b1);
-            segment<PLANE_XY>(q, b1, zhi);
-        }
-        segment<PLANE_Z>(q, zhi, nit);
-    }
-
-    template <int O>
-    __device__ __forceinline__ void shift(float4 (&q)[TY][QN])
-    {
+            for (int s = 0; s < 4; ++s) {
 #pragma unroll
-        for (int r = 0; r < TY; ++r)
-#pragma unroll
-            for (int jq = 0; jq < 8; ++jq) q[r][jq] = q[r][jq + O];
-    }
-
-    template <int O, int KIND>
-    __device__ __forceinline__ void group(float4 (&q)[TY][QN], int it)
-    {
-        if constexpr (O < U) {
-            plane<O, KIND>(q, it + O);
-            group<O + 1, KIND>(q, it);
-        }
-    }
-
-    // Iterations [it, it_end) of one kind (PML or interior): groups of U
-    // planes with compile-time queue offsets, then single planes.
-    template <int KIND>
-    __device__ __forceinline__ void segment(float4 (&q)[TY][QN], int it, int it_end)
-    {
-        if (U > 1) {
-            for (; it + U <= it_end && !aborted; it += U) {
-                group<0, KIND>(q, it);
-                shift<U>(q);
+                for (int r = 0; r < TY; ++r) q[r][4 * h + s] = E::ld(own_ptr(uf.off, r));
+                uf.next();
+            }
+            if (h == 0) {  // planes z0-4 .. z0-1 are not needed again
+                __syncwarp();
+                if ((tid & 31) == 0)
+#pragma unroll 1
+                    for (int s = 4; s >= 1; --s) mbar_arrive(empty_u(uf.behind(s)));
             }
         }
-        for (; it < it_end && !aborted; ++it) {
-            plane<0, KIND>(q, it);
-            shift<1>(q);
+        const int zlo = min(max(a.nb, z0), z1);
+        const int zhi = min(max(a.nb + a.nz, zlo), z1);
+        // The z-PML below the inner region, the planes between, the z-PML above: as a
+        // loop, so that each plane kind is compiled once (the kernel's code
+        // is far beyond the instruction cache of a scheduler either way).
+#pragma unroll 1
+        for (int part = 0; part < 3; ++part) {
+            const int k0 = part == 0 ? z0 : part == 1 ? zlo : zhi;
+            const int k1 = part == 0 ? zlo : part == 1 ? zhi : z1;
+            if (part != 1) {
+                segment<PLANE_Z>(q, k0, k1);
+            } else if constexpr (MODE != MODE_ADJ) {
+                if (xy_inner) segment<PLANE_INTERIOR>(q, k0, k1);
+                else segment<PLANE_XY>(q, k0, k1);
+            } else {  // the band planes next to the z-PML
+                const int b0 = xy_inner ? min(max(a.nb + BAND, k0), k1) : k1;
+                const int b1 = xy_inner ? min(max(a.nb + a.nz - BAND, b0), k1) : k1;
+#pragma unroll 1
+                for (int sub = 0; sub < 3; ++sub) {
+                    if (sub == 1) segment<PLANE_INTERIOR>(q, b0, b1);
+                    else segment<PLANE_XY>(q, sub == 0 ? k0 : b1, sub == 0 ? b0 : k1);
+                }
+            }
+        }
+    }
+
+    // Planes [k, k_end) of one kind.
+    template <int KIND>
+    __device__ __forceinline__ void segment(float4 (&q)[TY][QN], int k, int k_end)
+    {
+#pragma unroll 1
+        for (; k < k_end && !aborted; ++k) {
+            plane<KIND>(q, k);
+#pragma unroll
+            for (int r = 0; r < TY; ++r)
+#pragma unroll
+                for (int j = 0; j < QN - 1; ++j) q[r][j] = q[r][j + 1];
         }
     }
 };
@@ -1018,30 +1173,15 @@ __device__ __forceinline__ void step_unit(const StepArgs &a, int unit, int units
 {
     using S = StepCta<C, T, MODE, VAR>;
     constexpr bool SHELL = VAR == VAR_SHELL;
-    using G = Stage<C, T, MODE>;
     static_assert(MODE == MODE_FWD || MODE == MODE_DIFF || sizeof(T) == 4,
                   "the adjoint runs in fp32");
-    constexpr int TY = C::TY, NU = G::NU, NP = G::NP, THREADS = C::THREADS;
-    constexpr int BX = C::BX, BY = C::BY;
+    constexpr int TY = C::TY, THREADS = C::THREADS, BX = C::BX, BY = C::BY;
 
-    extern __shared__ __align__(128) unsigned char smem_raw[];
     S st;
     st.pa = &a;
-    st.su = smem_raw;
-    st.sp = smem_raw + NU * G::U_BYTES;
-    st.full_u = reinterpret_cast<uint64_t *>(st.sp + NP * G::P_BYTES + G::MZ_BYTES);
-    st.empty_u = st.full_u + NU;
-    st.full_p = st.empty_u + NU;
-    st.empty_p = st.full_p + NP;
-    st.lastf_u = reinterpret_cast<int *>(st.empty_p + NP);
-    st.lastf_p = st.lastf_u + NU;
-    // kept in the dynamic region: no static shared memory, so the TMA
-    // destinations start at the aligned base
-    st.s_abort = st.lastf_p + NP;
-
     const int tid = threadIdx.x;
     st.tid = tid;
-    st.lane = tid & 31;
+
 
     // Work unit: chunk-major so that CTAs running together share z and their
     // x-y halos meet in L2.
@@ -1071,17 +1211,7 @@ __device__ __forceinline__ void step_unit(const StepArgs &a, int unit, int units
     if (tid < THREADS) {
         if (!late) st.thread_geometry();
     } else if (tid == THREADS) {
-        *st.s_abort = 0;
-        for (int i = 0; i < NU; ++i) {
-            mbar_init(st.full_u + i, 1);
-            mbar_init(st.empty_u + i, C::WARPS);
-            st.lastf_u[i] = -1;
-        }
-        for (int i = 0; i < NP; ++i) {
-            mbar_init(st.full_p + i, 1);
-            mbar_init(st.empty_p + i, C::WARPS);
-            st.lastf_p[i] = -1;
-        }
+        st.init_rings(0);
         fence_barrier_init();
     }
     __syncthreads();
@@ -1166,12 +1296,12 @@ __device__ __forceinline__ void step_unit(const StepArgs &a, int unit, int units
     if constexpr (S::SCALED) {  // max |u^{n+1}| for the next step's scale
         float v = st.vmax;
         for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-        if (st.lane == 0 && v > 0.0f) atomicMax(reinterpret_cast<int *>(&a.scale->mx[(n + 1) & 3]),
+        if ((tid & 31) == 0 && v > 0.0f) atomicMax(reinterpret_cast<int *>(&a.scale->mx[(n + 1) & 3]),
                                                  __float_as_int(v));
         if constexpr (MODE == MODE_DIFF) {  // and max |d^{n+1}|
             float vd = st.vmax_d;
             for (int o = 16; o > 0; o >>= 1) vd = fmaxf(vd, __shfl_xor_sync(0xffffffffu, vd, o));
-            if (st.lane == 0 && vd > 0.0f)
+            if ((tid & 31) == 0 && vd > 0.0f)
                 atomicMax(reinterpret_cast<int *>(&a.scale_d->mx[(n + 1) & 3]), __float_as_int(vd));
         }
     }

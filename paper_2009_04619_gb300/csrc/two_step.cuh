@@ -142,7 +142,7 @@ struct TwoStepCta {
 
 // 25-point Laplacian of one quad in the interior path's operation order:
 // centre, z pairs (m = 1..4), y terms (m = 4..1 below, then 1..4 above), then
-// per point the x pairs.  q: z-queue with the centre at q[4]; rows(d): the quad
+// the x terms (lap_x).  q: z-queue with the centre at q[4]; rows(d): the quad
 // d rows away in the same plane (d = -4 .. 4, d != 0); lf, rt: the quads left
 // and right of the centre quad.
 template <class RowFn>
@@ -162,18 +162,7 @@ __device__ __forceinline__ float4 lap_quad(const TwoStepArgs &a, const float4 (&
         f4fma(L, a.cy[m - 1], rows(d));
     }
     const float4 c = q[4];
-    const float w[12] = {lf.x, lf.y, lf.z, lf.w, c.x, c.y, c.z, c.w, rt.x, rt.y, rt.z, rt.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        float s = f4get(L, e);
-#pragma unroll
-        for (int m = 1; m <= R; ++m) {
-            s = fmaf(a.cx[m - 1], w[4 + e - m], s);
-            s = fmaf(a.cx[m - 1], w[4 + e + m], s);
-        }
-        f4set(L, e, s);
-    }
-    return L;
+    return lap_x(L, a.cx, lf, c, rt);
 }
 
 template <class C>
