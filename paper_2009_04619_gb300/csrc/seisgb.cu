@@ -272,6 +272,28 @@ size_t align256(size_t b) { return (b + 255) / 256 * 256; }
 
 bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
+// fp32 weights of the three axes.  Rounded one by one they do not quite cancel
+// (c0 alone is off by up to 2^-28): a remainder that acts on u itself, 2e-6 of
+// k^2 u at 15 points per wavelength, and was most of a shot's error.  So w1 and
+// w2 of each axis may move by one unit in the last place (the outer ones, whose
+// relative accuracy sets the wavefield's leading tail, stay) until the 25 weights
+// add up to within a fraction of a unit of w2.
+void cancel_weights(float c0, float (&cx)[4], float (&cy)[4], float (&cz)[4])
+{
+    float *c[3] = {cx, cy, cz};
+    double sum = c0;
+    for (float *w : c)
+        for (int m = 0; m < 4; ++m) sum += 2.0 * w[m];
+    for (int m = 0; m < 2; ++m)
+        for (float *w : c) {
+            const double unit = std::nextafter(std::fabs(w[m]), INFINITY) - std::fabs(w[m]);
+            if (std::fabs(sum) <= unit) continue;  // a step of 2 units would not bring it nearer 0
+            const double d = sum > 0 ? -unit : unit;
+            w[m] = (float)(w[m] + d);
+            sum += 2.0 * d;
+        }
+}
+
 // Fill the parts of StepArgs that depend on the grid only.
 void fill_step_constants(const sgb_grid *g, const sgb_layout_info &L, StepArgs &a)
 {
@@ -294,6 +316,7 @@ void fill_step_constants(const sgb_grid *g, const sgb_layout_info &L, StepArgs &
         a.cy[m - 1] = (float)(W8[m] * iy);
         a.cz[m - 1] = (float)(W8[m] * iz);
     }
+    cancel_weights(a.c0, a.cx, a.cy, a.cz);
     // PML profile eta_a = eta_max_a (d / nb)^2, eta_max_a = -3 vmax ln r0 / (2 nb h_a)
     if (g->nb > 0 && g->pml_r0 < 1.0f) {
         const double nb = g->nb, dt = g->dt, lr = std::log((double)g->pml_r0);
