@@ -237,8 +237,8 @@ int run_shot_segment(const sgb_grid *g, const float *velocity, const float *wave
  * exact discrete adjoint of the fused step including the PML and the source
  * (the paper has no adjoint; the derivation is in the oracle and the design
  * notes).  The forward run keeps (u^n, u^{n-1}, phi^n) every ckpt_every steps
- * (0: 100); the backward sweep recomputes each segment's forward steps and
- * runs the adjoint steps over it.  The misfit sum is fp64; the time sum of the
+ * (0: 100); the backward sweep runs the adjoint steps segment by segment,
+ * recomputing each segment's forward steps but the last one's.  The misfit sum is fp64; the time sum of the
  * gradient is fp32 per point over blocks of 32 steps (counted from step 0, so
  * the result does not depend on ckpt_every) and fp64 across blocks;
  * everything else fp32 (SGB_FP32 storage only).
@@ -250,9 +250,9 @@ int run_shot_segment(const sgb_grid *g, const float *velocity, const float *wave
  * Calls on different streams (e.g. one host thread per stream) run
  * concurrently and independently: each call has its own scratch and its own
  * device error word.
- * Scratch: 9 padded fp32 fields and one fp64 field, ceil(nt / ckpt_every) x 3
- * checkpoint fields and
- * ckpt_every recomputation fields, from the library pool.  Synchronous. */
+ * Scratch: 9 padded fp32 fields and one fp64 field, 3 checkpoint fields for each
+ * of the ceil(nt / ckpt_every) segments but the first and the last, and
+ * ckpt_every fields of g, from the library pool.  Synchronous. */
 int adjoint_shot(const sgb_grid *g, const float *velocity, const float *wavelet, int32_t nt,
                  const int32_t *src_ijk, const int32_t *rec_ijk, int32_t nrec,
                  const float *observed, int32_t ckpt_every, double *misfit_out,
