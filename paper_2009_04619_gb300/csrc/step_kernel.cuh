@@ -270,9 +270,8 @@ struct Elem<__nv_bfloat16> {
     __device__ static __forceinline__ float4 ld(const __nv_bfloat16 *p)
     {
         const uint2 r = *reinterpret_cast<const uint2 *>(p);
-        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&r.x));
-        const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&r.y));
-        return make_float4(a.x, a.y, b.x, b.y);
+        return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xffff0000u),
+                           __uint_as_float(r.y << 16), __uint_as_float(r.y & 0xffff0000u));
     }
     __device__ static __forceinline__ __nv_bfloat162 pack(float x, float y, uint32_t rnd)
     {
