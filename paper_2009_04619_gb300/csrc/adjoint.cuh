@@ -27,7 +27,9 @@
 
 namespace {
 
-using CfgAdj = TileCfg<SGB_TXT, SGB_TYT, SGB_TY, SGB_NU, 2, SGB_MINB>;
+// The adjoint step's configuration for tile shape C: five tiles per plane, two stages.
+template <class C>
+using AdjCfg = TileCfg<C::TXT, C::TYT, C::TY, C::NU, 2, C::MINB>;
 constexpr int FOLD_EVERY = 32;
 
 // G += S, S = 0 over the padded arrays (the fp64 time sum of the gradient).
@@ -132,15 +134,19 @@ extern "C" int adjoint_shot(const sgb_grid *g, const float *velocity, const floa
     if ((rc = device_state(&ds))) return rc;
     if (!adjoint_prepared) {
         std::lock_guard<std::mutex> lk(g_mu);
-        CUDA_TRY(cudaFuncSetAttribute(fwd_acc_kernel<Cfg>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)Stage<Cfg, float, MODE_FWD_ACC>::SMEM_BYTES));
-        CUDA_TRY(cudaFuncSetAttribute(adjoint_step_kernel<CfgAdj>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)Stage<CfgAdj, float, MODE_ADJ>::SMEM_BYTES));
-        CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-            &adjoint_occ, adjoint_step_kernel<CfgAdj>, CfgAdj::BLOCK,
-            Stage<CfgAdj, float, MODE_ADJ>::SMEM_BYTES));
-        if (adjoint_occ < 1) return fail(SGB_ERR_CUDA, "adjoint step kernel does not fit on an SM");
+        int occ_acc = 0, occ_adj = 0;
+        for (const bool square : {false, true}) {
+            rc = with_tile(StepGrid{0, square}, [&](auto c) {
+                using C = decltype(c);
+                using A = AdjCfg<C>;
+                const int e = prepare_kernel<C>(fwd_acc_kernel<C>, Stage<C, float, MODE_FWD_ACC>::SMEM_BYTES,
+                                                &occ_acc);
+                return e ? e : prepare_kernel<A>(adjoint_step_kernel<A>, Stage<A, float, MODE_ADJ>::SMEM_BYTES,
+                                                 &occ_adj);
+            });
+            if (rc) return rc;
+        }
+        adjoint_occ = occ_adj;
         adjoint_prepared = 1;
     }
     cudaStream_t st = (cudaStream_t)stream;
@@ -199,12 +205,11 @@ extern "C" int adjoint_shot(const sgb_grid *g, const float *velocity, const floa
     base.sj = src_ijk[1];
     base.sk = src_ijk[2];
     base.wavelet = d_wav;
-    int grid = 0;
-    choose_decomposition(L.Nx, L.Ny, L.Nz, ds->sms, ds->occ, base, &grid);
+    const StepGrid sg = choose_decomposition<float>(ds->sms, ds->occ, base);
     float *ubuf[2] = {u0, u1};  // ubuf[0] = u^{-1}, ubuf[1] = u^0
     StepMaps fmaps[2];
     for (int p = 0; p < 2; ++p)
-        if ((rc = encode_step_maps<float>(fmaps[p], ubuf[(p + 1) & 1], ubuf[p & 1], m, phi, L))) return rc;
+        if ((rc = encode_step_maps<float>(fmaps[p], ubuf[(p + 1) & 1], ubuf[p & 1], m, phi, L, sg))) return rc;
 
     // 1. forward with checkpoints (u^n, u^{n-1}, phi^n before step n = s C).  The
     // last segment stores its g^n as it goes, so the backward sweep starts there
@@ -225,9 +230,12 @@ extern "C" int adjoint_shot(const sgb_grid *g, const float *velocity, const floa
             a.traces = d_tr;
         }
         const StepMaps &mp = fmaps[n & 1];
-        CUDA_TRY(launch_dependent(fwd_acc_kernel<Cfg>, grid, Cfg::BLOCK,
-                                  Stage<Cfg, float, MODE_FWD_ACC>::SMEM_BYTES, st, a, mp.ucur,
-                                  mp.ucur_in, mp.uprev, mp.m, mp.phi));
+        CUDA_TRY(with_tile(sg, [&](auto c) {
+            using C = decltype(c);
+            return launch_dependent(fwd_acc_kernel<C>, sg.ctas, C::BLOCK,
+                                    Stage<C, float, MODE_FWD_ACC>::SMEM_BYTES, st, a, mp.ucur,
+                                    mp.ucur_in, mp.uprev, mp.m, mp.phi);
+        }));
         ++t_launches;
         return SGB_OK;
     };
@@ -245,7 +253,7 @@ extern "C" int adjoint_shot(const sgb_grid *g, const float *velocity, const floa
         a.nrec = nrec;
         a.rec_off = d_off;
         a.traces = d_tr;
-        if ((rc = launch_step<float>(a, fmaps[n & 1], grid, st))) return rc;
+        if ((rc = launch_step<float>(a, fmaps[n & 1], sg, st))) return rc;
     }
     gather_kernel<<<(nrec + 255) / 256, 256, 0, st>>>(ubuf[(nt - 1) & 1], d_off, nrec,
                                                       d_tr + (size_t)(nt - 1) * nrec, d_err);
@@ -260,33 +268,34 @@ extern "C" int adjoint_shot(const sgb_grid *g, const float *velocity, const floa
     // 2. backward sweep, segment by segment from the last
     float *wbuf[2] = {w0, w1};  // w^k lives in wbuf[k & 1]
     float *mbuf[2] = {mu0, mu1};  // mu^k lives in mbuf[k & 1]
+    StepArgs abase = base;
+    abase.sk = -1;  // the adjoint's sources are the receivers
+    abase.gsum = gsum;
+    const StepGrid ag = choose_decomposition<float>(ds->sms, adjoint_occ, abase);
+    const int box_x = ag.square ? CfgSq::BX : Cfg::BX, box_y = ag.square ? CfgSq::BY : Cfg::BY;
     std::vector<CUtensorMap> acc_maps(C);
     for (int q = 0; q < C; ++q)
-        if ((rc = encode_map<float>(&acc_maps[q], seg + (size_t)q * L.elems, L, CfgAdj::BX, CfgAdj::BY)))
-            return rc;
+        if ((rc = encode_map<float>(&acc_maps[q], seg + (size_t)q * L.elems, L, box_x, box_y))) return rc;
     // [k & 1]: reads w^{k+1} = wbuf[(k+1)&1] and mu^{k+1}, writes wbuf[k&1]
     StepMaps amaps[2];
     for (int p = 0; p < 2; ++p) {
         if ((rc = encode_step_maps<float>(amaps[p], wbuf[(p + 1) & 1], wbuf[p & 1], m,
-                                          mbuf[(p + 1) & 1], L)))
+                                          mbuf[(p + 1) & 1], L, ag)))
             return rc;
         // mu^{k+1} as a box with its x-y neighbours (x halo 4, y halo 1)
-        using GA = Stage<CfgAdj, float, MODE_ADJ>;
-        if ((rc = encode_map<float>(&amaps[p].phi, mbuf[(p + 1) & 1], L, GA::MBW, GA::MBH, SGB_L2PROMO)))
-            return rc;
+        rc = with_tile(ag, [&](auto c) {
+            using GA = Stage<AdjCfg<decltype(c)>, float, MODE_ADJ>;
+            return encode_map<float>(&amaps[p].phi, mbuf[(p + 1) & 1], L, GA::MBW, GA::MBH, SGB_L2PROMO);
+        });
+        if (rc) return rc;
     }
     CUtensorMap gs_map;
-    if ((rc = encode_map<float>(&gs_map, gsum, L, CfgAdj::BX, CfgAdj::BY))) return rc;
-    StepArgs abase = base;
-    abase.sk = -1;  // the adjoint's sources are the receivers
-    abase.gsum = gsum;
-    int agrid = 0;
-    choose_decomposition(L.Nx, L.Ny, L.Nz, ds->sms, adjoint_occ, abase, &agrid);
+    if ((rc = encode_map<float>(&gs_map, gsum, L, box_x, box_y))) return rc;
     // receivers grouped by the unit that computes them
     UnitReceivers ur;
     int *d_rs, *d_ri;
     long long *d_ro;
-    group_receivers(abase, agrid, rec_ijk, nrec, ur);
+    with_tile(ag, [&](auto c) { group_receivers<decltype(c)>(abase, ag.ctas, rec_ijk, nrec, ur); });
     std::vector<long long> uoff(nrec);
     for (int q = 0; q < nrec; ++q) uoff[q] = off[ur.list[q]];
     if ((rc = sc.get((void **)&d_rs, ur.start.size() * 4)) || (rc = sc.get((void **)&d_ri, (size_t)nrec * 4)) ||
@@ -326,10 +335,13 @@ extern "C" int adjoint_shot(const sgb_grid *g, const float *velocity, const floa
             a.obs_row = d_obs + (size_t)(k - 1) * nrec;
             a.step_add = k;
             const StepMaps &mp = amaps[k & 1];
-            CUDA_TRY(launch_dependent(adjoint_step_kernel<CfgAdj>, agrid, CfgAdj::BLOCK,
-                                      Stage<CfgAdj, float, MODE_ADJ>::SMEM_BYTES, st, a, mp.ucur,
-                                      mp.ucur_in, mp.uprev, mp.m, mp.phi, acc_maps[k - 1 - na],
-                                      gs_map));
+            CUDA_TRY(with_tile(ag, [&](auto c) {
+                using A = AdjCfg<decltype(c)>;
+                return launch_dependent(adjoint_step_kernel<A>, ag.ctas, A::BLOCK,
+                                        Stage<A, float, MODE_ADJ>::SMEM_BYTES, st, a, mp.ucur,
+                                        mp.ucur_in, mp.uprev, mp.m, mp.phi, acc_maps[k - 1 - na],
+                                        gs_map);
+            }));
             ++t_launches;
             if ((k - 1) % FOLD_EVERY == 0) {  // blocks of steps counted from step 0
                 fold_kernel<<<fgrid, 256, 0, st>>>(gsum, gsum64, (long long)L.elems);

@@ -138,25 +138,35 @@ std::mutex g_mu;
 DevState g_dev[64];
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 
-// Allow the step kernel for storage T its dynamic shared memory; report how
-// many of its CTAs fit on one SM.
-template <class T, bool DIFF = false>
+template <class C, class T, bool DIFF = false>
 auto step_kernel_of()
 {
-    if constexpr (DIFF) return diff_step_kernel<Cfg, T>;
-    else return fused_step_kernel<Cfg, T>;
+    if constexpr (DIFF) return diff_step_kernel<C, T>;
+    else return fused_step_kernel<C, T>;
 }
 
+// Allow kernel kern of tiles C its dynamic shared memory; lower *occ to the
+// number of its CTAs that fit on one SM.
+template <class C, class K>
+int prepare_kernel(K kern, size_t smem, int *occ)
+{
+    int n = 0;
+    CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, C::BLOCK, smem));
+    if (n < 1) return fail(SGB_ERR_CUDA, "step kernel does not fit on an SM");
+    *occ = *occ > 0 ? std::min(*occ, n) : n;
+    return SGB_OK;
+}
+
+// ... the step kernels for storage T, both tile shapes
 template <class T, bool DIFF = false>
 int prepare_step_kernel(int *occ)
 {
-    using G = Stage<Cfg, T>;
-    const auto kern = step_kernel_of<T, DIFF>();
-    CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)G::SMEM_BYTES));
-    CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kern, Cfg::BLOCK, G::SMEM_BYTES));
-    if (*occ < 1) return fail(SGB_ERR_CUDA, "step kernel does not fit on an SM");
-    return SGB_OK;
+    *occ = 0;
+    int rc = prepare_kernel<Cfg>(step_kernel_of<Cfg, T, DIFF>(), Stage<Cfg, T>::SMEM_BYTES, occ);
+    if (!rc)
+        rc = prepare_kernel<CfgSq>(step_kernel_of<CfgSq, T, DIFF>(), Stage<CfgSq, T>::SMEM_BYTES, occ);
+    return rc;
 }
 
 int device_state(DevState **out)
@@ -375,25 +385,38 @@ struct StepMaps {
     CUtensorMap ucur, ucur_in, uprev, m, phi;
 };
 
-template <class T>
-int encode_step_maps(StepMaps &mp, const void *u_cur, const void *u_prev, const float *m,
+template <class C, class T>
+int encode_tile_maps(StepMaps &mp, const void *u_cur, const void *u_prev, const float *m,
                      const float *phi, const sgb_layout_info &L)
 {
-    using G = Stage<Cfg, T>;
+    using G = Stage<C, T>;
     int rc;
-    if ((rc = encode_map<T>(&mp.ucur, u_cur, L, G::SW, Cfg::SH, SGB_L2PROMO))) return rc;
-    if ((rc = encode_map<T>(&mp.ucur_in, u_cur, L, G::SW, Cfg::BY))) return rc;
-    if ((rc = encode_map<T>(&mp.uprev, u_prev, L, Cfg::BX, Cfg::BY))) return rc;
-    if ((rc = encode_map<float>(&mp.m, m, L, Cfg::BX, Cfg::BY))) return rc;
-    if ((rc = encode_map<float>(&mp.phi, phi ? phi : m, L, Cfg::PHI_BW, Cfg::BY))) return rc;
+    if ((rc = encode_map<T>(&mp.ucur, u_cur, L, G::SW, C::SH, SGB_L2PROMO))) return rc;
+    if ((rc = encode_map<T>(&mp.ucur_in, u_cur, L, G::SW, C::BY))) return rc;
+    if ((rc = encode_map<T>(&mp.uprev, u_prev, L, C::BX, C::BY))) return rc;
+    if ((rc = encode_map<float>(&mp.m, m, L, C::BX, C::BY))) return rc;
+    if ((rc = encode_map<float>(&mp.phi, phi ? phi : m, L, C::PHI_BW, C::BY))) return rc;
     return SGB_OK;
 }
 
-template <class T, bool DIFF = false>
-int launch_step(const StepArgs &a, const StepMaps &mp, int grid, cudaStream_t st)
+template <class T>
+int encode_step_maps(StepMaps &mp, const void *u_cur, const void *u_prev, const float *m,
+                     const float *phi, const sgb_layout_info &L, const StepGrid &sg)
 {
-    CUDA_TRY(launch_dependent(step_kernel_of<T, DIFF>(), grid, Cfg::BLOCK, Stage<Cfg, T>::SMEM_BYTES,
-                              st, a, mp.ucur, mp.ucur_in, mp.uprev, mp.m, mp.phi));
+    return with_tile(sg, [&](auto c) {
+        return encode_tile_maps<decltype(c), T>(mp, u_cur, u_prev, m, phi, L);
+    });
+}
+
+template <class T, bool DIFF = false>
+int launch_step(const StepArgs &a, const StepMaps &mp, const StepGrid &sg, cudaStream_t st)
+{
+    CUDA_TRY(with_tile(sg, [&](auto c) {
+        using C = decltype(c);
+        return launch_dependent(step_kernel_of<C, T, DIFF>(), sg.ctas, C::BLOCK,
+                                Stage<C, T>::SMEM_BYTES, st, a, mp.ucur, mp.ucur_in, mp.uprev, mp.m,
+                                mp.phi);
+    }));
     ++t_launches;
     return SGB_OK;
 }
@@ -699,11 +722,10 @@ int stencil_step_t(const sgb_grid *g, const sgb_layout_info &L, DevState *ds, cu
     const int occ = DIFF ? (std::is_same<T, float>::value ? ds->occ_df : ds->occ_db)
                     : std::is_same<T, float>::value ? ds->occ
                     : std::is_same<T, __half>::value ? ds->occ_h : ds->occ_b;
-    int grid = 0;
-    choose_decomposition(L.Nx, L.Ny, L.Nz, ds->sms, occ, a, &grid);
+    const StepGrid sg = choose_decomposition<T>(ds->sms, occ, a);
     StepMaps mp;
-    if ((rc = encode_step_maps<T>(mp, a.u_cur, DIFF ? d_io : a.u_out, m, phi, L))) return rc;
-    if ((rc = launch_step<T, DIFF>(a, mp, grid, st))) return rc;
+    if ((rc = encode_step_maps<T>(mp, a.u_cur, DIFF ? d_io : a.u_out, m, phi, L, sg))) return rc;
+    if ((rc = launch_step<T, DIFF>(a, mp, sg, st))) return rc;
     if (rec && rec->nrec > 0) {
         std::vector<long long> off(rec->nrec);
         for (int r = 0; r < rec->nrec; ++r)
@@ -923,8 +945,8 @@ int encode_pair_maps(PairMaps &pm, const float *a_prev, const float *b_cur, cons
     if ((rc = encode_map<float>(&pm.two_u, b_cur, L, TCfg::UW, TCfg::UH, SGB_L2PROMO))) return rc;
     if ((rc = encode_map<float>(&pm.two_up, a_prev, L, TCfg::EX, TCfg::EY))) return rc;
     if ((rc = encode_map<float>(&pm.two_m, m, L, TCfg::EX, TCfg::EY))) return rc;
-    if ((rc = encode_step_maps<float>(pm.shell0, b_cur, a_prev, m, phi, L))) return rc;
-    if ((rc = encode_step_maps<float>(pm.shell1, c_next, b_cur, m, phi, L))) return rc;
+    if ((rc = encode_tile_maps<Cfg, float>(pm.shell0, b_cur, a_prev, m, phi, L))) return rc;
+    if ((rc = encode_tile_maps<Cfg, float>(pm.shell1, c_next, b_cur, m, phi, L))) return rc;
     return SGB_OK;
 }
 
@@ -1026,6 +1048,7 @@ struct UnitReceivers {
     std::vector<int> start, list;
 };
 
+template <class C>
 void group_receivers(const StepArgs &a, int units, const int32_t *rec_ijk, int nrec, UnitReceivers &ur)
 {
     const int tiles = a.tiles_x * a.tiles_y;
@@ -1033,7 +1056,7 @@ void group_receivers(const StepArgs &a, int units, const int32_t *rec_ijk, int n
     ur.list.assign(std::max(nrec, 1), 0);
     auto unit_of = [&](int r) {
         const int i = rec_ijk[3 * r], j = rec_ijk[3 * r + 1], k = rec_ijk[3 * r + 2];
-        return (k / a.zc) * tiles + (j / Cfg::BY) * a.tiles_x + i / Cfg::BX;
+        return (k / a.zc) * tiles + (j / C::BY) * a.tiles_x + i / C::BX;
     };
     for (int r = 0; r < nrec; ++r) ++ur.start[unit_of(r) + 1];
     for (int u = 0; u < units; ++u) ur.start[u + 1] += ur.start[u];
@@ -1066,7 +1089,7 @@ int run_flow(const sgb_layout_info &L, DevState *ds, cudaStream_t st, Scratch &s
     }
     const int chunks = (L.Nz + fa.zc - 1) / fa.zc, units = tiles * chunks;
     UnitReceivers ur;
-    group_receivers(fa, units, rec_ijk, nrec, ur);
+    group_receivers<Cfg>(fa, units, rec_ijk, nrec, ur);
     const std::vector<int> &rs = ur.start, &rl = ur.list;
     int *d_done, *d_counter, *d_rs, *d_rl;
     if ((rc = sc.get((void **)&d_done, (size_t)units * 4)) || (rc = sc.get((void **)&d_counter, 16)) ||
@@ -1180,17 +1203,18 @@ int run_shot_t(const sgb_grid *g, const sgb_layout_info &L, DevState *ds, cudaSt
                                                              : ds->occ_db)
                     : std::is_same<T, float>::value ? ds->occ
                     : std::is_same<T, __half>::value ? ds->occ_h : ds->occ_b;
-    int grid = 0;
-    choose_decomposition(L.Nx, L.Ny, L.Nz, ds->sms, occ, base, &grid);
+    StepGrid sg = choose_decomposition<T>(ds->sms, occ, base);
+    const bool flow = !Elem<T>::SCALED && !DIFF && resolve_schedule(g) == SGB_SCHED_FLOW && nsteps > 0;
+    if (flow) sg.square = false;  // the dataflow kernel has units of its own, of 64 x 16 tiles
     StepMaps maps[2];  // [parity of n]; the difference form reads d^n through the u^{n-1} map
     for (int p = 0; p < 2; ++p)
         if ((rc = encode_step_maps<T>(maps[p], buf[(p + 1) & 1], DIFF ? dfield : buf[p & 1], m, phi,
-                                      L)))
+                                      L, sg)))
             return rc;
 
     bool looped = false;
     if constexpr (!Elem<T>::SCALED && !DIFF) {
-        if (resolve_schedule(g) == SGB_SCHED_FLOW && nsteps > 0) {
+        if (flow) {
             if ((rc = run_flow<T>(L, ds, st, sc, base, maps, buf, n_begin, n_end, rec_ijk, nrec)))
                 return rc;
             looped = true;
@@ -1207,7 +1231,7 @@ int run_shot_t(const sgb_grid *g, const sgb_layout_info &L, DevState *ds, cudaSt
             a.u_out = buf[n & 1];
             a.u_cur = buf[(n + 1) & 1];
             a.step_add = n;
-            if ((rc = launch_step<T, DIFF>(a, maps[n & 1], grid, st))) return rc;
+            if ((rc = launch_step<T, DIFF>(a, maps[n & 1], sg, st))) return rc;
         }
 
     // u^k lives in buf[(k+1)&1] (written by step k-1): u^{nt} in buf[(nt+1)&1]
@@ -1335,11 +1359,10 @@ int run_shot_pairs(const sgb_grid *g, const sgb_layout_info &L, DevState *ds, cu
         a.u_out = u[2 * par];
         a.u_cur = u[2 * par + 1];
         a.step_add = n;
-        int grid = 0;
-        choose_decomposition(L.Nx, L.Ny, L.Nz, ds->sms, ds->occ, a, &grid);
+        const StepGrid sg = choose_decomposition<float>(ds->sms, ds->occ, a);
         StepMaps mp;
-        if ((rc = encode_step_maps<float>(mp, a.u_cur, a.u_out, m, phi, L))) return rc;
-        if ((rc = launch_step<float>(a, mp, grid, st))) return rc;
+        if ((rc = encode_step_maps<float>(mp, a.u_cur, a.u_out, m, phi, L, sg))) return rc;
+        if ((rc = launch_step<float>(a, mp, sg, st))) return rc;
         u_final_dev = u[2 * par];
     }
     if (nrec > 0 && nt > 0) {
@@ -1769,18 +1792,17 @@ extern "C" int run_shot_noalloc(const sgb_grid *g, const float *velocity, const 
     base_args.nrec = nrec;
     base_args.rec_off = d_off;
     base_args.traces = traces;
-    int grid = 0;
-    choose_decomposition(L.Nx, L.Ny, L.Nz, ns->sms, ns->occ, base_args, &grid);
+    const StepGrid sg = choose_decomposition<float>(ns->sms, ns->occ, base_args);
     StepMaps maps[2];
     for (int p = 0; p < 2; ++p)
-        if ((rc = encode_step_maps<float>(maps[p], buf[(p + 1) & 1], buf[p & 1], m, phi, L))) return rc;
+        if ((rc = encode_step_maps<float>(maps[p], buf[(p + 1) & 1], buf[p & 1], m, phi, L, sg))) return rc;
     for (int n = 0; n < nt; ++n) {
         StepArgs a = base_args;
         a.u_out = buf[n & 1];
         a.u_cur = buf[(n + 1) & 1];
         a.step_ptr = nullptr;
         a.step_add = n;
-        if ((rc = launch_step<float>(a, maps[n & 1], grid, st))) return rc;
+        if ((rc = launch_step<float>(a, maps[n & 1], sg, st))) return rc;
     }
     float *u_last = nt > 0 ? buf[(nt - 1) & 1] : buf[1];
     if (nrec > 0 && nt > 0) {

@@ -69,7 +69,7 @@ struct Shot {
     int *d_step = nullptr;  // this shot's device step counter (step of a replay's first launch)
     StepArgs args;          // step constants, fields, source, receivers, decomposition
     StepMaps maps[2];       // [parity of n]
-    int grid = 0;           // work units per step
+    StepGrid grid;          // work units per step, tile shape
     int n0 = 0;             // next step to run
     Clock::time_point t_submit, t_admit, t_done;
 };
@@ -217,10 +217,11 @@ int setup_shot(sgb_server *sv, Shot *sh)
     a.rec_off = sh->d_off;
     a.traces = sh->d_tr;
     // the shot's own decomposition, as run_shot would choose it
-    choose_decomposition(L.Nx, L.Ny, L.Nz, sv->ds->sms, sv->ds->occ, a, &sh->grid);
+    sh->grid = choose_decomposition<float>(sv->ds->sms, sv->ds->occ, a);
     float *buf[2] = {sh->u0, sh->u1};  // buf[0] = u^{-1}, buf[1] = u^0
     for (int p = 0; p < 2; ++p)  // step n reads buf[(n+1)&1], writes buf[n&1]
-        if ((rc = encode_step_maps<float>(sh->maps[p], buf[(p + 1) & 1], buf[p & 1], sh->m, sh->phi, L)))
+        if ((rc = encode_step_maps<float>(sh->maps[p], buf[(p + 1) & 1], buf[p & 1], sh->m, sh->phi, L,
+                                          sh->grid)))
             return rc;
     sh->n0 = 0;
     return SGB_OK;
@@ -286,10 +287,13 @@ int prepare_replay(sgb_server *sv)
                 r.step_ptr = sh->d_step;
                 r.step_add = k;
                 r.n_end = sh->nt;
-                ce = launch_dependent(shot_step_kernel<Cfg>, sh->grid, Cfg::BLOCK,
-                                      Stage<Cfg, float>::SMEM_BYTES, bs, sh->args, r, p0.ucur,
-                                      p0.ucur_in, p0.uprev, p0.m, p0.phi, p1.ucur, p1.ucur_in,
-                                      p1.uprev, p1.m, p1.phi);
+                ce = with_tile(sh->grid, [&](auto c) {
+                    using C = decltype(c);
+                    return launch_dependent(shot_step_kernel<C>, sh->grid.ctas, C::BLOCK,
+                                            Stage<C, float>::SMEM_BYTES, bs, sh->args, r, p0.ucur,
+                                            p0.ucur_in, p0.uprev, p0.m, p0.phi, p1.ucur,
+                                            p1.ucur_in, p1.uprev, p1.m, p1.phi);
+                });
             }
             if (ce == cudaSuccess) {
                 advance_kernel<<<1, 32, 0, bs>>>(sh->d_step, S);
@@ -466,8 +470,10 @@ extern "C" int serve_create(const sgb_serve_config *cfg, sgb_server **out)
     DevState *ds;
     int rc = device_state(&ds);
     if (rc) return rc;
-    CUDA_TRY(cudaFuncSetAttribute(shot_step_kernel<Cfg>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)Stage<Cfg, float>::SMEM_BYTES));
+    int occ = 0;
+    if ((rc = prepare_kernel<Cfg>(shot_step_kernel<Cfg>, Stage<Cfg, float>::SMEM_BYTES, &occ)) ||
+        (rc = prepare_kernel<CfgSq>(shot_step_kernel<CfgSq>, Stage<CfgSq, float>::SMEM_BYTES, &occ)))
+        return rc;
     sgb_server *sv = new sgb_server();
     sv->cfg = *cfg;
     sv->ds = ds;

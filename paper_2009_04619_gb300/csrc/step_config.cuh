@@ -4,6 +4,8 @@
 #pragma once
 #include <cuda.h>
 
+#include <algorithm>
+
 #include "step_kernel.cuh"
 
 namespace sgb {
@@ -40,47 +42,101 @@ namespace sgb {
 #ifndef SGB_L2PROMO_P
 #define SGB_L2PROMO_P CU_TENSOR_MAP_L2_PROMOTION_NONE
 #endif
+// Two tile shapes of as many points: 64 x 16, whose rows are whole 256-byte
+// lines, and 32 x 32.  choose_decomposition takes one of them per grid.
 using Cfg = TileCfg<SGB_TXT, SGB_TYT, SGB_TY, SGB_NU, SGB_NP, SGB_MINB>;
+using CfgSq = TileCfg<SGB_TXT / 2, 2 * SGB_TYT, SGB_TY, SGB_NU, SGB_NP, SGB_MINB>;
 
-// Chunking of z: pick the chunk length that minimises waves x (chunk + priming
-// overhead) for the resident-CTA slots of this GPU.  Chunks are capped at 40
-// planes: CTAs of tiles in the x-y PML band move 1.5x the bytes per plane of
-// interior tiles, so neighbours drift apart in z over long chunks and their
-// shared halos fall out of L2 (measured on 512^3: 22-40-plane chunks move ~10%
-// fewer DRAM bytes than 74-plane chunks; with the 9-stage u^n ring 40-plane
-// chunks ran 1.7% faster than 27-plane ones, 52- and 64-plane chunks slower).
-inline void choose_decomposition(int Nx, int Ny, int Nz, int sms, int occ, StepArgs &a, int *grid)
+// How a step of one grid is launched (the tile counts and zc are in StepArgs).
+struct StepGrid {
+    int ctas = 0;
+    bool square = false;  // CfgSq instead of Cfg
+};
+
+// f(C{}) with the grid's tile configuration.
+template <class F>
+auto with_tile(const StepGrid &sg, F f)
 {
-    a.tiles_x = (Nx + Cfg::BX - 1) / Cfg::BX;
-    a.tiles_y = (Ny + Cfg::BY - 1) / Cfg::BY;
-    const long long tiles = (long long)a.tiles_x * a.tiles_y;
-    const long long slots = (long long)sms * occ;
-    int best_zc = Nz;
-    double best = 1e300;
-#ifdef SGB_FORCE_CHUNKS
-    {
-        const int zc = (Nz + SGB_FORCE_CHUNKS - 1) / SGB_FORCE_CHUNKS;
-        a.zc = zc;
-        *grid = (int)(tiles * ((Nz + zc - 1) / zc));
-        return;
-    }
-#endif
-    const int cmax = Nz / 4 > 1 ? Nz / 4 : 1;
-    for (int c = 1; c <= cmax; ++c) {
-        const int zc = (Nz + c - 1) / c;
-        if (zc > 40 && c < cmax) continue;
-        const int ceff = (Nz + zc - 1) / zc;
-        const long long units = tiles * ceff;
-        const long long waves = (units + slots - 1) / slots;
-        const double cost = (double)waves * (zc + 8 * 0.5);
-        if (cost < best * 0.999) {
-            best = cost;
-            best_zc = zc;
-        }
-    }
-    a.zc = best_zc;
-    *grid = (int)(tiles * ((Nz + best_zc - 1) / best_zc));
+    return sg.square ? f(CfgSq{}) : f(Cfg{});
 }
 
+// Estimated time of one step with tiles C and the z-chunk length that minimises
+// it, in planes of an interior tile per CTA slot: waves x (chunk + 4 planes of
+// priming) x (1 + 0.2 x the share of tile planes in the PML).  With 16-bit storage
+// a partly filled wave after a full one counts half: CTAs of different cost refill
+// their slots as they finish (400^3 bf16: 201 us with the 40 planes it then takes,
+// 204 with 25; in fp32 a whole wave is the better guess, 343 x 229 x 205: 76 us with
+// 21 planes, 77.5 with 35).  Alone in one wave, the dearest CTA decides.  Chunks of 64 x 16
+// and 16-bit tiles have at most 40 planes: neighbouring CTAs drift apart in z
+// over longer ones and their shared halos fall out of L2 (512^3: 22-40-plane
+// chunks move ~10% fewer DRAM bytes than 74-plane ones).  The fp32 32 x 32 tiles
+// have twice the row ends per point and lose more to it (512^3: 414 us with 40
+// planes, 405 with 24): 30 planes, or 36 in a single wave.
+template <class C, class T>
+double plan_chunks(const StepArgs &a, int slots, int *zc_out)
+{
+    constexpr double part = sizeof(T) == 4 ? 1.0 : 0.5;  // a partly filled wave
+    constexpr bool short_chunks = C::BX < Cfg::BX && sizeof(T) == 4;
+    const int tx = (a.Nx + C::BX - 1) / C::BX, ty = (a.Ny + C::BY - 1) / C::BY;
+    const int tiles = tx * ty;
+    double pml = 0.0, pml_one = 0.0;  // PML share of all tile planes; of the dearest CTA's
+    if (a.nb > 0) {
+        const int ix = std::max((a.Nx - a.nb) / C::BX - (a.nb + C::BX - 1) / C::BX, 0);
+        const int iy = std::max((a.Ny - a.nb) / C::BY - (a.nb + C::BY - 1) / C::BY, 0);
+        const double zshare = std::min(1.0, 2.0 * a.nb / a.Nz);
+        const double xy = 1.0 - double(ix) * iy / tiles;
+        pml = xy + (1.0 - xy) * zshare;
+        pml_one = xy > 0.0 ? 1.0 : zshare;
+    }
+    const int cmax = std::max(a.Nz / 4, 1);
+    double best = 1e300;
+    *zc_out = a.Nz;
+    int last = 0;
+    for (int c = 1; c <= cmax; ++c) {
+        const int zc = (a.Nz + c - 1) / c;
+        if (zc == last) continue;
+        last = zc;
+        const int units = tiles * ((a.Nz + zc - 1) / zc);
+        const bool one = units <= slots;
+        if (zc > (short_chunks ? (one ? 36 : 30) : 40) && c < cmax) continue;
+        const double w = double(units) / slots;
+        const double waves = one ? 1.0 : w + part * ((units + slots - 1) / slots - w);
+        const double cost = waves * (zc + 4) * (1.0 + 0.2 * (one ? pml_one : pml));
+        if (cost < best * 0.999) {
+            best = cost;
+            *zc_out = zc;
+        }
+    }
+    return best;
+}
+
+// Tile shape and z-chunks of a step kernel for storage T with occ resident CTAs
+// per SM.  Which shape is faster is a matter of how the extents divide: 64 x 16
+// spends 22% of its points outside a 200-wide grid, 32 x 32 covers less of a PML
+// 16 to 32 points wide with its dearer edge tiles, and either may fit one wave
+// where the other needs two.  Where both divide evenly, 32 x 32 costs fp32 4%
+// (row ends: 256^3 60.4 -> 62.0 us) and 16-bit storage nothing.  On 23 grids from
+// 96^3 to 512^3 the estimate's choice is within 3% of the faster shape at its
+// best chunk length, 0.7% on average (PML 10-32, us, 64 x 16 -> 32 x 32: fp32
+// 160^3 18.8 -> 16.8, 200^3 39.8 -> 34.7; bf16 200^3 42.9 -> 37.2, 224^3 49.7 ->
+// 41.8, 282^3 91.9 -> 81.6, 352^3 145 -> 131, 512^3 376 -> 365).
+template <class T>
+StepGrid choose_decomposition(int sms, int occ, StepArgs &a)
+{
+    const int slots = sms * occ;
+    int zc = 0, zc_sq = 0;
+    const double wide = plan_chunks<Cfg, T>(a, slots, &zc);
+    const double square = plan_chunks<CfgSq, T>(a, slots, &zc_sq) * (sizeof(T) == 4 ? 1.04 : 1.0);
+    StepGrid sg;
+    sg.square = square < wide;
+    a.zc = sg.square ? zc_sq : zc;
+    with_tile(sg, [&](auto c) {
+        using C = decltype(c);
+        a.tiles_x = (a.Nx + C::BX - 1) / C::BX;
+        a.tiles_y = (a.Ny + C::BY - 1) / C::BY;
+    });
+    sg.ctas = a.tiles_x * a.tiles_y * ((a.Nz + a.zc - 1) / a.zc);
+    return sg;
+}
 
 }  // namespace sgb
