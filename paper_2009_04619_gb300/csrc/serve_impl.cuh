@@ -9,7 +9,8 @@
 // - The scheduler thread admits queued requests in FIFO order while a slot is
 //   free and the budget holds the head's footprint, sets their fields up on a
 //   second stream while the current replays run, and advances every resident
-//   shot with replays of one CUDA graph.  The graph has one branch per resident
+//   shot with replays of one CUDA graph, or with the same launches enqueued one by
+//   one where a capture would cost more.  A replay has one branch per resident
 //   shot: steps_per_graph launches of the fused step on that shot's own grid
 //   and decomposition (arguments and tensor maps in the kernel's parameter
 //   space, as in run_shot), then an increment of the shot's device step
@@ -21,7 +22,7 @@
 //   repeats.  A shot of nt steps takes nt + 1 launches (the last samples the
 //   receivers of the last step); launches past that return at once.
 // - Composition changes (admission, retirement) happen between replays; the
-//   graph is re-captured only then.  Retired shots' traces are copied to the
+//   graph is re-captured only after one.  Retired shots' traces are copied to the
 //   host and their device memory returned to the pool.
 // - The host enqueues several replays back to back and waits only where the
 //   composition can change: up to the next shot completion when no request can
@@ -259,8 +260,44 @@ int retire_shot(sgb_server *sv, Shot *sh)
     return rc;
 }
 
-// (Re)capture the replay graph when the composition changed: one branch per
-// resident shot with steps_per_graph launches and the counter increment.
+// One replay onto stream cs (or into its capture): a branch per resident shot with
+// steps_per_graph launches, step by step over the shots so that none waits for
+// another's to be enqueued, and the counter increment.
+cudaError_t enqueue_replay(sgb_server *sv, cudaStream_t cs)
+{
+    const int S = sv->cfg.steps_per_graph;
+    const size_t n = sv->resident.size();
+    cudaError_t ce = cudaEventRecord(sv->ev_fork, cs);
+    for (size_t i = 0; i < n && ce == cudaSuccess; ++i)
+        ce = cudaStreamWaitEvent(sv->branch[i], sv->ev_fork, 0);
+    for (int k = 0; k < S; ++k)
+        for (size_t i = 0; i < n && ce == cudaSuccess; ++i) {
+            Shot *sh = sv->resident[i];
+            const StepMaps &p0 = sh->maps[0], &p1 = sh->maps[1];
+            ShotRun r;
+            r.buf[0] = sh->u0;
+            r.buf[1] = sh->u1;
+            r.step_ptr = sh->d_step;
+            r.step_add = k;
+            r.n_end = sh->nt;
+            ce = with_tile(sh->grid, [&](auto c) {
+                using C = decltype(c);
+                return launch_dependent(shot_step_kernel<C>, sh->grid.ctas, C::BLOCK,
+                                        Stage<C, float>::SMEM_BYTES, sv->branch[i], sh->args, r,
+                                        p0.ucur, p0.ucur_in, p0.uprev, p0.m, p0.phi, p1.ucur,
+                                        p1.ucur_in, p1.uprev, p1.m, p1.phi);
+            });
+        }
+    for (size_t i = 0; i < n && ce == cudaSuccess; ++i) {
+        advance_kernel<<<1, 32, 0, sv->branch[i]>>>(sv->resident[i]->d_step, S);
+        ce = cudaGetLastError();
+        if (ce == cudaSuccess) ce = cudaEventRecord(sv->ev_join[i], sv->branch[i]);
+        if (ce == cudaSuccess) ce = cudaStreamWaitEvent(cs, sv->ev_join[i], 0);
+    }
+    return ce;
+}
+
+// (Re)capture the replay graph when the composition changed.
 int prepare_replay(sgb_server *sv)
 {
     if (!sv->composition_changed && sv->exec) return SGB_OK;
@@ -268,40 +305,12 @@ int prepare_replay(sgb_server *sv)
         cudaGraphExecDestroy(sv->exec);
         sv->exec = nullptr;
     }
-    const int S = sv->cfg.steps_per_graph;
     cudaStream_t cs;
     CUDA_TRY(cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking));
     cudaGraph_t graph = nullptr;
     cudaError_t ce = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
     if (ce == cudaSuccess) {
-        ce = cudaEventRecord(sv->ev_fork, cs);
-        for (size_t i = 0; i < sv->resident.size() && ce == cudaSuccess; ++i) {
-            Shot *sh = sv->resident[i];
-            cudaStream_t bs = sv->branch[i];
-            ce = cudaStreamWaitEvent(bs, sv->ev_fork, 0);
-            const StepMaps &p0 = sh->maps[0], &p1 = sh->maps[1];
-            for (int k = 0; k < S && ce == cudaSuccess; ++k) {
-                ShotRun r;
-                r.buf[0] = sh->u0;
-                r.buf[1] = sh->u1;
-                r.step_ptr = sh->d_step;
-                r.step_add = k;
-                r.n_end = sh->nt;
-                ce = with_tile(sh->grid, [&](auto c) {
-                    using C = decltype(c);
-                    return launch_dependent(shot_step_kernel<C>, sh->grid.ctas, C::BLOCK,
-                                            Stage<C, float>::SMEM_BYTES, bs, sh->args, r, p0.ucur,
-                                            p0.ucur_in, p0.uprev, p0.m, p0.phi, p1.ucur,
-                                            p1.ucur_in, p1.uprev, p1.m, p1.phi);
-                });
-            }
-            if (ce == cudaSuccess) {
-                advance_kernel<<<1, 32, 0, bs>>>(sh->d_step, S);
-                ce = cudaGetLastError();
-            }
-            if (ce == cudaSuccess) ce = cudaEventRecord(sv->ev_join[i], bs);
-            if (ce == cudaSuccess) ce = cudaStreamWaitEvent(cs, sv->ev_join[i], 0);
-        }
+        ce = enqueue_replay(sv, cs);
         cudaError_t ee = cudaStreamEndCapture(cs, &graph);
         if (ce == cudaSuccess) ce = ee;
     }
@@ -311,6 +320,21 @@ int prepare_replay(sgb_server *sv)
     CUDA_TRY(ce);
     sv->composition_changed = false;
     return SGB_OK;
+}
+
+// Whether a few replays of a new composition are better enqueued launch by launch
+// than captured first: the GPU stands still while a graph is captured and
+// instantiated (0.15 ms for 16 steps of six shots, at each admission and
+// retirement), and a launch costs the host 3 us, so the resident shots' steps must
+// take the GPU longer than that on average.  A CTA plane takes it about 0.8 us.
+// Six requests of 128^3 to 128 x 128 x 176, 100 steps: 7.5 -> 6.2-6.6 ms.
+bool enqueue_directly(const sgb_server *sv, int replays)
+{
+    if (replays > MAX_AHEAD_OPEN || (!sv->composition_changed && sv->exec)) return false;
+    double gpu_us = 0.0;
+    for (const Shot *sh : sv->resident) gpu_us += 0.8 * sh->grid.ctas * (sh->args.zc + 4);
+    gpu_us /= std::max(sv->ds->sms * sv->ds->occ, 1);
+    return gpu_us >= 4.0 * sv->resident.size();
 }
 
 void scheduler(sgb_server *sv)
@@ -352,10 +376,13 @@ void scheduler(sgb_server *sv)
         Clock::time_point tp = Clock::now();
         double t_prep = 0.0, t_setup = 0.0, t_wait = 0.0, t_retire = 0.0;
         if (replay) {
-            rc = prepare_replay(sv);
+            const bool direct = enqueue_directly(sv, R);
+            if (!direct) rc = prepare_replay(sv);
             t_prep = ms_between(tp, Clock::now());
             for (int r = 0; r < R && rc == SGB_OK && e == cudaSuccess; ++r)
-                e = cudaGraphLaunch(sv->exec, sv->stream);
+                e = direct ? enqueue_replay(sv, sv->stream) : cudaGraphLaunch(sv->exec, sv->stream);
+            if (direct && e != cudaSuccess)  // branches that the stream does not wait for
+                for (size_t i = 0; i < sv->resident.size(); ++i) cudaStreamSynchronize(sv->branch[i]);
             t_launches += (int64_t)R * (S + 1) * (int64_t)sv->resident.size();
         }
         tp = Clock::now();
