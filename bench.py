@@ -42,8 +42,8 @@ HBM_FALLBACK_GBS = 6800.0
 # kernel source it was measured on (comments and whitespace removed); a
 # changed kernel reports null.
 NCU_TRAFFIC = {
-    # ncu on the 512^3 + 32-point-PML step: 1.959 GB read + 0.678 GB written per launch
-    "c661d56f6bfa4b42": 2.638e9,
+    # ncu on the 512^3 + 32-point-PML step: 1.958 GB read + 0.678 GB written per launch
+    "e40ea65592144ab3": 2.635e9,
 }
 
 
@@ -464,7 +464,7 @@ def _small_case(a, seisgb, synth, dev, barrier):
     return {"workload": w.name, "grid": list(w.shape), "nt": w.nt, "value": w.points * w.nt / ms / 1e6,
             "unit": UNIT, "ms_per_shot": ms,
             "note": "fields fit in L2 (4 x 4.5 MB): no roofline claim; includes run_shot's per-call "
-                    "set-up (allocation, m, velocity range check, graph capture)"}
+                    "set-up (allocation, m, velocity range check)"}
 
 
 def run_reference(a):

@@ -289,16 +289,16 @@ int run_shot_noalloc(const sgb_grid *g, const float *velocity, const float *wave
  * current device at serve_create), a stream and a scheduler thread.  Requests
  * are admitted in FIFO order whenever a slot is free and the server's HBM
  * budget can hold their footprint; all resident shots, whatever their grid
- * sizes, advance together in replays of one CUDA graph that holds, for every
- * resident shot, a branch of steps_per_graph fused-step launches on that shot's
- * own grid; the branches run concurrently on the GPU.  Shots join and leave
- * between graph replays.  A shot's results equal run_shot's for the same
- * request, bit for bit.
+ * sizes, advance together in replays that hold, for every resident shot, a
+ * branch of steps_per_graph fused-step launches on that shot's own grid (one CUDA
+ * graph, or the launches by themselves while the composition keeps changing); the
+ * branches run concurrently on the GPU.  Shots join and leave between replays.
+ * A shot's results equal run_shot's for the same request, bit for bit.
  * ------------------------------------------------------------------------- */
 typedef struct {
     uint64_t hbm_budget_bytes;  /* device memory the resident shots may hold */
     int32_t max_slots;          /* shots resident at once, 1..64 */
-    int32_t steps_per_graph;    /* time steps per CUDA-graph replay, 1..256 */
+    int32_t steps_per_graph;    /* time steps per replay, 1..256 */
 } sgb_serve_config;
 
 typedef struct {
@@ -333,9 +333,8 @@ typedef struct {
     uint64_t graph_replays, step_launches;
     uint64_t device_bytes;      /* bytes held by resident shots */
     /* scheduler-thread time (ms, cumulative): setting up admitted shots (host
-     * side; their copies overlap the running replays), uploading the shot
-     * table and re-capturing the replay graph, retiring finished shots, and
-     * waiting for enqueued replays to finish */
+     * side; their copies overlap the running replays), re-capturing the replay
+     * graph, retiring finished shots, and waiting for enqueued replays to finish */
     double setup_ms, prepare_ms, retire_ms, wait_ms;
     uint64_t cancelled;         /* requests ended by serve_cancel */
 } sgb_serve_stats;

@@ -52,8 +52,10 @@
 //    polled at once, the x taps and the PML update are packed pairs, and each
 //    plane kind is compiled once (83 -> 46 KB of code).  Per step, before and
 //    after: 512^3 + PML 32 411 -> 403 us, 256^3 + PML 16 63.1 -> 61.5 us, 96^3
-//    7.6 -> 7.2 us; bf16 at 512^3 427 -> 399 us, fp16 at 384 x 384 x 256 143 -> 132
-//    us.  No register may spill: beside 2 x 113 KB of shared memory the L1 holds
+//    7.6 -> 7.2 us; bf16 at 512^3 427 -> 362 us and fp16 at 384 x 384 x 256 143 -> 126
+//    us, with bf16 pairs unpacked by shift and mask (-13 us), no spilled values
+//    (-10 us) and 32 x 32 tiles (-11 us), the bf16 figures.  No register may spill:
+//    beside 2 x 113 KB of shared memory the L1 holds
 //    a few KB, and a spilled value read in the z loop comes from L2 (80 bytes of
 //    spills took 256^3 from 65 to 95 us);
 //  - eta and its central differences are evaluated in closed form from the
@@ -1144,8 +1146,9 @@ __device__ __forceinline__ float pow2_scale_for(float B)
     return ldexpf(1.0f, ilogbf(B) + 1 - 14);
 }
 
-// Resident CTAs per SM asked of the compiler: 16-bit storage halves the u
-// ring's shared memory, leaving room for a third CTA if registers allow.
+// Resident CTAs per SM asked of the compiler, also for 16-bit storage: its shared
+// memory would leave room for a third CTA, but 128 registers a thread do not hold
+// the z-queue (spills, 9-27% slower).
 template <class C, class T>
 constexpr int min_blocks()
 {
@@ -1180,7 +1183,6 @@ __device__ __forceinline__ void step_unit(const StepArgs &a, int unit, int units
     st.pa = &a;
     const int tid = threadIdx.x;
     st.tid = tid;
-
 
     // Work unit: chunk-major so that CTAs running together share z and their
     // x-y halos meet in L2.
@@ -1354,7 +1356,7 @@ __global__ void __launch_bounds__(C::BLOCK, C::MINB)
     });
 }
 
-// One step of one shot inside a CUDA-graph replay: the step n = *step_ptr +
+// One step of one shot in a served replay: the step n = *step_ptr +
 // step_add comes from a device counter, the buffers and tensor maps of its
 // parity are chosen here (so a replay of any length repeats), and launches past
 // the shot's last step do nothing (n_end: the last launch, which only samples
