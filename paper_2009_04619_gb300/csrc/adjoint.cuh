@@ -83,8 +83,10 @@ __global__ void misfit_final_kernel(const double *partial, double *J)
 
 // dJ/dv = 2 (sum_k w^k g^{k-1}) / v on the compact grid, planes in grid.y.  fp64
 // division is slow here (87 us at 128^3): 1 / v comes from the fp32 reciprocal
-// and one Newton step in fp64 (relative error below 2^-46), the indices from one
-// 32-bit division.
+// and one Newton step in fp64 (relative error below 2^-46), the quotient from a
+// product and its residual (Markstein, IBM J. Res. Dev. 34, 1990), which leaves an
+// error of half a unit in the last place, as the division did; the indices come
+// from one 32-bit division.
 __global__ void chain_kernel(PadGeom g, const double *__restrict__ G,
                              const float *__restrict__ vel, double *__restrict__ grad_v)
 {
@@ -97,7 +99,9 @@ __global__ void chain_kernel(PadGeom g, const double *__restrict__ G,
             double inv = (double)__frcp_rn(v);
             inv = fma(inv, fma(-(double)v, inv, 1.0), inv);
             if (!(v > 1e-30f && v < 1e30f)) inv = 1.0 / (double)v;  // no fp32 reciprocal there
-            grad_v[c0 + t] = 2.0 * G[p0 + j * g.sx + i] * inv;
+            const double num = 2.0 * G[p0 + j * g.sx + i], quo = num * inv;
+            // an infinite quotient has no residual
+            grad_v[c0 + t] = isfinite(quo) ? fma(fma(-(double)v, quo, num), inv, quo) : quo;
         }
     }
 }
