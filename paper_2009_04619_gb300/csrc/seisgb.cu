@@ -722,7 +722,7 @@ int stencil_step_t(const sgb_grid *g, const sgb_layout_info &L, DevState *ds, cu
     const int occ = DIFF ? (std::is_same<T, float>::value ? ds->occ_df : ds->occ_db)
                     : std::is_same<T, float>::value ? ds->occ
                     : std::is_same<T, __half>::value ? ds->occ_h : ds->occ_b;
-    const StepGrid sg = choose_decomposition<T>(ds->sms, occ, a);
+    const StepGrid sg = choose_decomposition<T, DIFF>(ds->sms, occ, a);
     StepMaps mp;
     if ((rc = encode_step_maps<T>(mp, a.u_cur, DIFF ? d_io : a.u_out, m, phi, L, sg))) return rc;
     if ((rc = launch_step<T, DIFF>(a, mp, sg, st))) return rc;
@@ -1203,7 +1203,7 @@ int run_shot_t(const sgb_grid *g, const sgb_layout_info &L, DevState *ds, cudaSt
                                                              : ds->occ_db)
                     : std::is_same<T, float>::value ? ds->occ
                     : std::is_same<T, __half>::value ? ds->occ_h : ds->occ_b;
-    StepGrid sg = choose_decomposition<T>(ds->sms, occ, base);
+    StepGrid sg = choose_decomposition<T, DIFF>(ds->sms, occ, base);
     const bool flow = !Elem<T>::SCALED && !DIFF && resolve_schedule(g) == SGB_SCHED_FLOW && nsteps > 0;
     if (flow) sg.square = false;  // the dataflow kernel has units of its own, of 64 x 16 tiles
     StepMaps maps[2];  // [parity of n]; the difference form reads d^n through the u^{n-1} map

@@ -119,14 +119,23 @@ double plan_chunks(const StepArgs &a, int slots, int *zc_out)
 // 96^3 to 512^3 the estimate's choice is within 3% of the faster shape at its
 // best chunk length, 0.7% on average (PML 10-32, us, 64 x 16 -> 32 x 32: fp32
 // 160^3 18.8 -> 16.8, 200^3 39.8 -> 34.7; bf16 200^3 42.9 -> 37.2, 224^3 49.7 ->
-// 41.8, 282^3 91.9 -> 81.6, 352^3 145 -> 131, 512^3 376 -> 365).
-template <class T>
+// 41.8, 282^3 91.9 -> 81.6, 352^3 145 -> 131, 512^3 376 -> 365).  The fp32
+// difference form moves a fifth more bytes, and a single wave of 32 x 32 tiles loses
+// more to its row ends there once the chunks are long (64 x 16 -> 32 x 32: 157 x
+// 215 x 193 39.3 -> 41.8 us, 144 x 256 x 176 33.0 -> 35.5, 150 x 169 x 309 45.5 ->
+// 48.6 with 25 to 31 planes; 224 x 208 x 160 42.1 -> 41.2, the estimate 16% apart;
+// 146 x 126 x 135 17.6 -> 14.5 and 129 x 87 x 171 14.9 -> 12.8 with 9): 15% there.
+template <class T, bool DIFF = false>
 StepGrid choose_decomposition(int sms, int occ, StepArgs &a)
 {
     const int slots = sms * occ;
     int zc = 0, zc_sq = 0;
     const double wide = plan_chunks<Cfg, T>(a, slots, &zc);
-    const double square = plan_chunks<CfgSq, T>(a, slots, &zc_sq) * (sizeof(T) == 4 ? 1.04 : 1.0);
+    double square = plan_chunks<CfgSq, T>(a, slots, &zc_sq);
+    const long long units_sq = (long long)((a.Nx + CfgSq::BX - 1) / CfgSq::BX) *
+                               ((a.Ny + CfgSq::BY - 1) / CfgSq::BY) * ((a.Nz + zc_sq - 1) / zc_sq);
+    const bool long_wave = DIFF && zc_sq > 16 && units_sq <= slots;
+    square *= sizeof(T) == 2 ? 1.0 : long_wave ? 1.15 : 1.04;
     StepGrid sg;
     sg.square = square < wide;
     a.zc = sg.square ? zc_sq : zc;
