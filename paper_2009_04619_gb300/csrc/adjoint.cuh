@@ -88,11 +88,12 @@ __global__ void misfit_final_kernel(const double *partial, double *J)
 // error of half a unit in the last place, as the division did; the indices come
 // from one 32-bit division.
 __global__ void chain_kernel(PadGeom g, const double *__restrict__ G,
-                             const float *__restrict__ vel, double *__restrict__ grad_v)
+                             const float *__restrict__ vel, double *__restrict__ grad_v, int j0,
+                             int rows)
 {
-    const uint32_t items = uint32_t(g.Nx) * uint32_t(g.Ny);
+    const uint32_t items = uint32_t(g.Nx) * uint32_t(rows);
     for (int k = blockIdx.y; k < g.Nz; k += gridDim.y) {
-        const long long c0 = (long long)k * items, p0 = g.origin + k * g.sxy;
+        const long long c0 = ((long long)k * g.Ny + j0) * g.Nx, p0 = g.origin + k * g.sxy + j0 * g.sx;
         for (uint32_t t = blockIdx.x * blockDim.x + threadIdx.x; t < items; t += gridDim.x * blockDim.x) {
             const uint32_t j = t / uint32_t(g.Nx), i = t - j * uint32_t(g.Nx);
             const float v = vel[c0 + t];
@@ -358,9 +359,10 @@ extern "C" int adjoint_shot(const sgb_grid *g, const float *velocity, const floa
     double *d_gv = grad_velocity;
     const bool host_gv = !is_device_ptr(grad_velocity);
     if (host_gv && (rc = sc.get((void **)&d_gv, (size_t)ncomp * 8))) return rc;
-    chain_kernel<<<conv_grid((long long)L.Nx * L.Ny, L.Nz), CONV_THREADS, 0, st>>>(pad_geom(L), gsum64,
-                                                                                 d_vel, d_gv);
-    CUDA_TRY(cudaGetLastError());
+    CUDA_TRY(for_row_slabs(L.Ny, L.Nx, [&](int j0, int rows) {
+        chain_kernel<<<conv_grid((long long)L.Nx * rows, L.Nz), CONV_THREADS, 0, st>>>(
+            pad_geom(L), gsum64, d_vel, d_gv, j0, rows);
+    }));
     if (host_gv)
         CUDA_TRY(cudaMemcpyAsync(grad_velocity, d_gv, (size_t)ncomp * 8, cudaMemcpyDeviceToHost, st));
     double J = 0.0;

@@ -19,7 +19,9 @@ struct PadGeom {
 // flat index took most of the time before), and each thread has CONV_UNROLL
 // loads in flight before its first store.  384 x 384 x 256: pack 222 -> 51 us,
 // unpack 124 -> 49 us (323 and 302 MB: 6.3 and 6.1 TB/s); 383 x 381 x 257, point
-// by point: 220 -> 77 and 122 -> 60 us.
+// by point: 220 -> 77 and 122 -> 60 us.  The items that one launch counts in a
+// plane fit 32 bits: rows j0 .. j0 + rows - 1 of every plane, all of them but in
+// planes of more than 2^31 items (for_row_slabs).
 constexpr int CONV_THREADS = 256, CONV_UNROLL = 4, CONV_ITEMS = CONV_THREADS * CONV_UNROLL;
 
 // Items of V elements: global loads and stores (fp32 and 16-bit).
@@ -71,22 +73,23 @@ __device__ __forceinline__ void st_vec(T *p, const Vec<1> &q)
 template <class T, int V, bool M>
 __global__ void __launch_bounds__(CONV_THREADS)
     to_padded_kernel(PadGeom g, const float *__restrict__ src, T *__restrict__ dst, float dt,
-                     int *range)
+                     int *range, int j0, int rows)
 {
-    const uint32_t row = uint32_t(g.sx) / V, items = row * uint32_t(g.sxy / g.sx);
+    const uint32_t row = uint32_t(g.sx) / V, items = row * uint32_t(rows);
     float mx = 0.0f, mn = 3.0e38f;
     int bad = 0;
     for (int kk = blockIdx.y; kk < g.Nz + 8; kk += gridDim.y) {
         const bool in_z = kk >= 4 && kk < g.Nz + 4;
         const float *sp = src + (long long)(kk - 4) * g.Ny * g.Nx;
-        T *dp = dst + (long long)kk * g.sxy;
+        T *dp = dst + (long long)kk * g.sxy + j0 * g.sx;
         const uint32_t t0 = blockIdx.x * CONV_ITEMS + threadIdx.x;
         Vec<V> val[CONV_UNROLL];
 #pragma unroll
         for (int u = 0; u < CONV_UNROLL; ++u) {
             const uint32_t t = t0 + u * CONV_THREADS;
-            const int jj = t / row, ii = (t - jj * row) * V;
-            const int i = ii - 8, j = jj - 4;
+            const uint32_t jj = t / row;
+            const int ii = (t - jj * row) * V;
+            const int i = ii - 8, j = j0 + int(jj) - 4;
             const bool in = t < items && in_z && i >= 0 && i < g.Nx && j >= 0 && j < g.Ny;
 #pragma unroll
             for (int e = 0; e < V; ++e) val[u].v[e] = 0.0f;
@@ -140,13 +143,13 @@ __global__ void __launch_bounds__(CONV_THREADS)
 template <class T, int V>
 __global__ void __launch_bounds__(CONV_THREADS)
     from_padded_kernel(PadGeom g, const T *__restrict__ src, const float *scale,
-                       float *__restrict__ dst)
+                       float *__restrict__ dst, int j0, int rows)
 {
-    const uint32_t row = uint32_t(g.Nx) / V, items = row * uint32_t(g.Ny);
+    const uint32_t row = uint32_t(g.Nx) / V, items = row * uint32_t(rows);
     const float s = scale ? *scale : 1.0f;
     for (int k = blockIdx.y; k < g.Nz; k += gridDim.y) {
-        const T *sp = src + g.origin + (long long)k * g.sxy;
-        float *dp = dst + (long long)k * g.Ny * g.Nx;
+        const T *sp = src + g.origin + (long long)k * g.sxy + j0 * g.sx;
+        float *dp = dst + ((long long)k * g.Ny + j0) * g.Nx;
         const uint32_t t0 = blockIdx.x * CONV_ITEMS + threadIdx.x;
         Vec<V> val[CONV_UNROLL];
 #pragma unroll

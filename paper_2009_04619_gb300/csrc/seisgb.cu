@@ -440,6 +440,21 @@ dim3 conv_grid(long long plane_items, int planes)
                 (unsigned)std::min(planes, 65535));
 }
 
+// launch(j0, rows) over the rows of a plane, in slabs of at most 2^31 items (one but
+// for planes of tens of thousands of points either way), and its status.
+template <class F>
+cudaError_t for_row_slabs(long long rows, long long row_items, F launch)
+{
+    const long long most = std::max(1LL, (1LL << 31) / row_items);
+    cudaError_t e = cudaSuccess;
+    for (long long j0 = 0; j0 < rows && e == cudaSuccess; j0 += most) {
+        launch((int)j0, (int)std::min(most, rows - j0));
+        ++t_launches;
+        e = cudaGetLastError();
+    }
+    return e;
+}
+
 // Whether rows of a compact array can be moved as quads.
 bool quad_rows(const sgb_layout_info &L, const void *compact, const void *padded)
 {
@@ -451,14 +466,16 @@ template <class T, bool M = false>
 cudaError_t enqueue_to_padded(const sgb_layout_info &L, const float *src, T *dst, cudaStream_t st,
                               float dt = 0.0f, int *range = nullptr)
 {
-    if (quad_rows(L, src, dst))
-        to_padded_kernel<T, 4, M><<<conv_grid(L.stride_z / 4, (int)L.sz), CONV_THREADS, 0, st>>>(
-            pad_geom(L), src, dst, dt, range);
-    else
-        to_padded_kernel<T, 1, M><<<conv_grid(L.stride_z, (int)L.sz), CONV_THREADS, 0, st>>>(
-            pad_geom(L), src, dst, dt, range);
-    ++t_launches;
-    return cudaGetLastError();
+    const int V = quad_rows(L, src, dst) ? 4 : 1;
+    return for_row_slabs(L.sy, L.sx / V, [&](int j0, int rows) {
+        const dim3 grid = conv_grid(L.sx / V * rows, (int)L.sz);
+        if (V == 4)
+            to_padded_kernel<T, 4, M><<<grid, CONV_THREADS, 0, st>>>(pad_geom(L), src, dst, dt, range, j0,
+                                                                     rows);
+        else
+            to_padded_kernel<T, 1, M><<<grid, CONV_THREADS, 0, st>>>(pad_geom(L), src, dst, dt, range, j0,
+                                                                     rows);
+    });
 }
 
 // padded T -> compact fp32, times *scale (null: 1).
@@ -466,15 +483,14 @@ template <class T>
 cudaError_t enqueue_from_padded(const sgb_layout_info &L, const T *src, const float *scale, float *dst,
                                 cudaStream_t st)
 {
-    const long long plane = (long long)L.Nx * L.Ny;
-    if (quad_rows(L, dst, src))
-        from_padded_kernel<T, 4><<<conv_grid(plane / 4, L.Nz), CONV_THREADS, 0, st>>>(pad_geom(L), src,
-                                                                                     scale, dst);
-    else
-        from_padded_kernel<T, 1><<<conv_grid(plane, L.Nz), CONV_THREADS, 0, st>>>(pad_geom(L), src,
-                                                                                 scale, dst);
-    ++t_launches;
-    return cudaGetLastError();
+    const int V = quad_rows(L, dst, src) ? 4 : 1;
+    return for_row_slabs(L.Ny, L.Nx / V, [&](int j0, int rows) {
+        const dim3 grid = conv_grid((long long)(L.Nx / V) * rows, L.Nz);
+        if (V == 4)
+            from_padded_kernel<T, 4><<<grid, CONV_THREADS, 0, st>>>(pad_geom(L), src, scale, dst, j0, rows);
+        else
+            from_padded_kernel<T, 1><<<grid, CONV_THREADS, 0, st>>>(pad_geom(L), src, scale, dst, j0, rows);
+    });
 }
 
 int ew_grid(long long n, const DevState &ds)
