@@ -243,7 +243,8 @@ int run_shot_segment(const sgb_grid *g, const float *velocity, const float *wave
  * the result does not depend on ckpt_every) and fp64 across blocks;
  * everything else fp32 (SGB_FP32 storage only).
  *   velocity  Nz*Ny*Nx fp32 compact, host or device
- *   wavelet   nt fp32, host or device;  src_ijk, rec_ijk: host
+ *   wavelet   nt fp32, host or device;  src_ijk, rec_ijk: host (receivers may
+ *             share a point: each adds its residual)
  *   observed  nt*nrec fp32 (same layout as run_shot's traces), host or device
  *   misfit_out     host double
  *   grad_velocity  Nz*Ny*Nx fp64 compact, host or device

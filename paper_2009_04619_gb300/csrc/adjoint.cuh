@@ -296,11 +296,17 @@ extern "C" int adjoint_shot(const sgb_grid *g, const float *velocity, const floa
     }
     CUtensorMap gs_map;
     if ((rc = encode_map<float>(&gs_map, gsum, L, box_x, box_y))) return rc;
-    // receivers grouped by the unit that computes them
+    // receivers grouped by the unit that computes them, and in a unit by point (the
+    // residuals of receivers at one point are added by one thread)
     UnitReceivers ur;
     int *d_rs, *d_ri;
     long long *d_ro;
     with_tile(ag, [&](auto c) { group_receivers<decltype(c)>(abase, ag.ctas, rec_ijk, nrec, ur); });
+    const auto by_point = [&](int p, int q) { return off[p] < off[q]; };
+    for (int u = 0; u < ag.ctas; ++u) {
+        const auto r0 = ur.list.begin() + ur.start[u], r1 = ur.list.begin() + ur.start[u + 1];
+        if (!std::is_sorted(r0, r1, by_point)) std::stable_sort(r0, r1, by_point);
+    }
     std::vector<long long> uoff(nrec);
     for (int q = 0; q < nrec; ++q) uoff[q] = off[ur.list[q]];
     if ((rc = sc.get((void **)&d_rs, ur.start.size() * 4)) || (rc = sc.get((void **)&d_ri, (size_t)nrec * 4)) ||
