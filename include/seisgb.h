@@ -291,9 +291,10 @@ int run_shot_noalloc(const sgb_grid *g, const float *velocity, const float *wave
  * are admitted in FIFO order whenever a slot is free and the server's HBM
  * budget can hold their footprint; all resident shots, whatever their grid
  * sizes, advance together in replays that hold, for every resident shot, a
- * branch of steps_per_graph fused-step launches on that shot's own grid (one CUDA
- * graph, or the launches by themselves while the composition keeps changing); the
- * branches run concurrently on the GPU.  Shots join and leave between replays.
+ * branch of steps_per_graph fused-step launches on that shot's own grid: one CUDA
+ * graph, or the launches by themselves for the first replays after shots joined or
+ * left and for those that only lead up to the next change; the branches run
+ * concurrently on the GPU.  Shots join and leave between replays.
  * A shot's results equal run_shot's for the same request, bit for bit.
  * ------------------------------------------------------------------------- */
 typedef struct {
@@ -331,7 +332,8 @@ typedef struct {
 typedef struct {
     uint64_t submitted, completed, rejected;
     int32_t resident, queued;
-    uint64_t graph_replays, step_launches;
+    uint64_t graph_replays;     /* replays of a captured graph */
+    uint64_t step_launches;     /* steps_per_graph for each replay, captured or not */
     uint64_t device_bytes;      /* bytes held by resident shots */
     /* scheduler-thread time (ms, cumulative): setting up admitted shots (host
      * side; their copies overlap the running replays), re-capturing the replay

@@ -10,7 +10,7 @@
 //   free and the budget holds the head's footprint, sets their fields up on a
 //   second stream while the current replays run, and advances every resident
 //   shot with replays of one CUDA graph, or with the same launches enqueued one by
-//   one where a capture would cost more.  A replay has one branch per resident
+//   one where a capture would cost more (enqueue_directly).  A replay has one branch per resident
 //   shot: steps_per_graph launches of the fused step on that shot's own grid
 //   and decomposition (arguments and tensor maps in the kernel's parameter
 //   space, as in run_shot), then an increment of the shot's device step
@@ -22,7 +22,8 @@
 //   repeats.  A shot of nt steps takes nt + 1 launches (the last samples the
 //   receivers of the last step); launches past that return at once.
 // - Composition changes (admission, retirement) happen between replays; the
-//   graph is re-captured only after one.  Retired shots' traces are copied to the
+//   graph is re-captured only after one, once the new composition has outlived its
+//   first batch of replays.  Retired shots' traces are copied to the
 //   host and their device memory returned to the pool.
 // - The host enqueues several replays back to back and waits only where the
 //   composition can change: up to the next shot completion when no request can
@@ -42,6 +43,7 @@ namespace {
 constexpr int SERVE_MAX_SLOTS = 64;
 constexpr int MAX_AHEAD_OPEN = 4;     // replays enqueued at once while slots are free
 constexpr int MAX_AHEAD_FULL = 256;   // ... while every slot is taken
+constexpr int MAX_DIRECT = 8;         // a composition of at most so many more is not captured
 
 using Clock = std::chrono::steady_clock;
 
@@ -134,6 +136,7 @@ struct sgb_server {
     // the graph of the current composition: one branch (stream) per resident shot
     cudaGraphExec_t exec = nullptr;
     bool composition_changed = true;
+    int direct_replays = 0;  // replays enqueued launch by launch since it changed
     cudaStream_t branch[SERVE_MAX_SLOTS] = {};
     cudaEvent_t ev_fork = nullptr, ev_join[SERVE_MAX_SLOTS] = {};
 };
@@ -322,15 +325,19 @@ int prepare_replay(sgb_server *sv)
     return SGB_OK;
 }
 
-// Whether a few replays of a new composition are better enqueued launch by launch
-// than captured first: the GPU stands still while a graph is captured and
-// instantiated (0.15 ms for 16 steps of six shots, at each admission and
-// retirement), and a launch costs the host 3 us, so the resident shots' steps must
-// take the GPU longer than that on average.  A CTA plane takes it about 0.8 us.
-// Six requests of 128^3 to 128 x 128 x 176, 100 steps: 7.5 -> 6.2-6.6 ms.
-bool enqueue_directly(const sgb_server *sv, int replays)
+// Whether the next replays are better enqueued launch by launch than captured first:
+// the GPU stands still while a graph is captured and instantiated (0.15 ms for 16
+// steps of six shots), and a launch costs the host 3 us, so the resident shots' steps
+// must take the GPU longer than that on average.  A CTA plane takes it about 0.8 us.
+// A graph saves about 0.7 us a step at 128^3 (one shot 10.7 -> 10.0 us a step, four
+// 10.7 -> 9.7), so it repays its capture after some ten replays: those of a composition
+// that has outlived a first batch and will not end within to_finish <= MAX_DIRECT
+// replays are captured.  Six requests of 128^3 to 128 x 128 x 176, 100 steps: 7.5 ms
+// with every composition captured, 6.2-6.6 ms so.
+bool enqueue_directly(const sgb_server *sv, int replays, int to_finish)
 {
     if (replays > MAX_AHEAD_OPEN || (!sv->composition_changed && sv->exec)) return false;
+    if (sv->direct_replays > 0 && to_finish > MAX_DIRECT) return false;
     double gpu_us = 0.0;
     for (const Shot *sh : sv->resident) gpu_us += 0.8 * sh->grid.ctas * (sh->args.zc + 4);
     gpu_us /= std::max(sv->ds->sms * sv->ds->occ, 1);
@@ -366,18 +373,19 @@ void scheduler(sgb_server *sv)
         cudaError_t e = cudaSuccess;
         const bool replay = !sv->resident.empty();
         int R = 1;
+        int to_finish = MAX_AHEAD_FULL;  // replays until the first resident shot is done
+        for (Shot *sh : sv->resident)
+            to_finish = std::min(to_finish, std::max(1, (sh->nt + 1 - sh->n0 + S - 1) / S));
         if (replay && admit.empty()) {
-            int to_finish = MAX_AHEAD_FULL;  // replays until the first resident shot is done
-            for (Shot *sh : sv->resident)
-                to_finish = std::min(to_finish, std::max(1, (sh->nt + 1 - sh->n0 + S - 1) / S));
             const bool open = (int)sv->resident.size() < sv->cfg.max_slots;
             R = open ? std::min(to_finish, MAX_AHEAD_OPEN) : to_finish;
         }
         Clock::time_point tp = Clock::now();
         double t_prep = 0.0, t_setup = 0.0, t_wait = 0.0, t_retire = 0.0;
+        const bool direct = replay && enqueue_directly(sv, R, to_finish);
         if (replay) {
-            const bool direct = enqueue_directly(sv, R);
-            if (!direct) rc = prepare_replay(sv);
+            if (direct) sv->direct_replays += R;
+            else rc = prepare_replay(sv);
             t_prep = ms_between(tp, Clock::now());
             for (int r = 0; r < R && rc == SGB_OK && e == cudaSuccess; ++r)
                 e = direct ? enqueue_replay(sv, sv->stream) : cudaGraphLaunch(sv->exec, sv->stream);
@@ -434,12 +442,15 @@ void scheduler(sgb_server *sv)
             }
         }
         for (Shot *sh : finished) retire_shot(sv, sh);
-        if (!finished.empty() || !joined.empty()) sv->composition_changed = true;
+        if (!finished.empty() || !joined.empty()) {
+            sv->composition_changed = true;
+            sv->direct_replays = 0;
+        }
         t_retire = ms_between(tp, Clock::now());
         {
             std::lock_guard<std::mutex> lk(sv->mu);
             if (replay) {
-                sv->stats.graph_replays += R;
+                if (!direct) sv->stats.graph_replays += R;
                 sv->stats.step_launches += (uint64_t)R * S;
             }
             sv->stats.prepare_ms += t_prep;
