@@ -136,7 +136,9 @@ int sgb_cfl_dt(const sgb_grid *g, float vmax, float *dt_max);
  * difference-form formats through stencil_step_diff (INVALID_ARG here).  step
  * selects src->wavelet[step].
  * src and rec may be NULL.  All device pointers must be 16-byte aligned.
- * Asynchronous on stream.  UNSTABLE_DT when g->dt exceeds the CFL limit for
+ * Asynchronous on stream.  A stream capture may hold any number of steps without
+ * receivers (their points are read from rec->ijk during the call, so a replay would
+ * not find them).  UNSTABLE_DT when g->dt exceeds the CFL limit for
  * g->vmax.  A bounded kernel wait that gave up or a non-finite receiver sample
  * sets a bit of this device's stencil_step error word, which
  * sgb_device_status reads and clears. */
